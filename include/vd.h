@@ -39,7 +39,8 @@
  *   to about 1e-12 of the data's scale.  Every score's rounding error is
  *   relative to the score itself (a few 1e-7 in practice).  Ranking: a NaN
  *   score ranks below every number, +0 and -0 are equal.
- * - Launches: one eviction kernel per call, plus a one-thread-per-sequence
+ * - Launches: one eviction kernel per call (calls of few units take one that
+ *   keeps a unit's scored rows in shared memory), plus a one-thread-per-sequence
  *   length update (a programmatic dependent launch of the eviction, all on
  *   `stream`).  A hole-fill block eviction or a score-only call that fits
  *   one wave at one CTA per unit but has more units than the GPU has SMs

@@ -15,6 +15,7 @@
 
 #include "vd.h"
 #include "vd_evict.cuh"
+#include "vd_resident.cuh"
 #include "vd_small.cuh"
 
 namespace vd {
@@ -24,6 +25,9 @@ const void* evict_kernel_norm(bool decode, bool holefill, bool fused);
 const void* small_kernel_l2(bool decode, bool fused);
 const void* small_kernel_dir(bool decode, bool fused);
 const void* small_kernel_norm(bool decode, bool fused);
+const void* resident_kernel_l2(bool decode, bool fused);
+const void* resident_kernel_dir(bool decode, bool fused);
+const void* resident_kernel_norm(bool decode, bool fused);
 const void* score_kernel_l2();
 const void* score_kernel_dir();
 const void* score_kernel_norm();
@@ -166,6 +170,14 @@ const void* small_kernel(vd_variant var, bool decode, bool fused) {
   }
 }
 
+const void* resident_kernel(vd_variant var, bool decode, bool fused) {
+  switch (var) {
+    case VD_SCORE_L2: return vd::resident_kernel_l2(decode, fused);
+    case VD_SCORE_DIR: return vd::resident_kernel_dir(decode, fused);
+    default: return vd::resident_kernel_norm(decode, fused);
+  }
+}
+
 vd_status device_state(DeviceState** out) {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) {
@@ -201,10 +213,11 @@ vd_status device_state(DeviceState** out) {
           return VD_ERR_CUDA;
       }
     for (int var = 0; var < 3; ++var)
-      for (int kind = 0; kind < 5; ++kind) {
-        const void* kern = kind == 4 ? score_kernel((vd_variant)var)
-                                     : small_kernel((vd_variant)var, (kind & 1) != 0,
-                                                    (kind & 2) != 0);
+      for (int kind = 0; kind < 9; ++kind) {
+        const bool dec = (kind & 1) != 0, fus = (kind & 2) != 0;
+        const void* kern = kind == 8  ? score_kernel((vd_variant)var)
+                           : kind < 4 ? small_kernel((vd_variant)var, dec, fus)
+                                      : resident_kernel((vd_variant)var, dec, fus);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  st.smem_optin) != cudaSuccess ||
             cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
@@ -236,8 +249,17 @@ int lanes_per_row(int d) {
   return p;
 }
 
-bool cluster_fits(const void* kern, long long groups, int c, size_t smem) {
-  if (c == 1) return true;
+// How many clusters of c CTAs (of kThreads threads) run at once.
+long long active_clusters(const void* kern, long long groups, int c, size_t smem,
+                          const DeviceState& st) {
+  int n = 0;
+  if (c == 1) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, kThreads, smem) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
+    }
+    return (long long)n * st.sms;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(groups * c));
   cfg.blockDim = dim3(kThreads);
@@ -249,12 +271,16 @@ bool cluster_fits(const void* kern, long long groups, int c, size_t smem) {
   attr.val.clusterDim.z = 1;
   cfg.attrs = &attr;
   cfg.numAttrs = 1;
-  int ncl = 0;
-  if (cudaOccupancyMaxActiveClusters(&ncl, kern, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return 0;
   }
-  return ncl > 0;
+  return n;
+}
+
+bool cluster_fits(const void* kern, long long groups, int c, size_t smem,
+                  const DeviceState& st) {
+  return c == 1 || active_clusters(kern, groups, c, smem, st) > 0;
 }
 
 bool cluster_allowed(int c, int d) {
@@ -303,7 +329,7 @@ int choose_cluster(const void* kern, long long units, int d, int capacity, int k
       cudaGetLastError();
       continue;
     }
-    if (occ < 1 || !cluster_fits(kern, units, c, smem)) continue;
+    if (occ < 1 || !cluster_fits(kern, units, c, smem, st)) continue;
     if (want < 1 && !cluster_allowed(c, d)) {
       // narrower row segments than preferred: only when nothing else fits
       // (a large capacity at a small head dim)
@@ -377,7 +403,7 @@ long long split_plan(const void* kern, long long units, int d, int capacity, int
     if (solo + joint * c > P * occ) continue;  // one wave
     const double load = (double)((solo + P - 1) / P) + (double)((joint * c + P - 1) / P) / c;
     const size_t smem_c = vd::smem_layout(capacity, c, kind).total;
-    if (load < best && cluster_fits(kern, joint, c, smem_c)) {
+    if (load < best && cluster_fits(kern, joint, c, smem_c, st)) {
       best = load;
       best_solo = solo;
       *c_out = c;
@@ -451,8 +477,6 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
 // forms, block and decode, take the same kernel.
 constexpr size_t kSmallRowBytes = 64 * 1024;
 
-bool cluster_fits(const void* kern, long long groups, int c, size_t smem);
-
 bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* weights,
                const float* disp_out, int score_k, const DeviceState& st) {
   if (score_only || holefill || weights || disp_out || score_k) return false;
@@ -482,7 +506,7 @@ bool cached_fits(const void* kern, long long groups, int c, size_t smem, DeviceS
         return e.c != 0;
     }
   }
-  const bool fits = c == 1 || cluster_fits(kern, groups, c, smem);
+  const bool fits = cluster_fits(kern, groups, c, smem, st);
   std::lock_guard<std::mutex> lk(g_mu);
   st.choice[st.next_choice] =
       ClusterChoice{kern, groups, 0, 0, kFitsKind, c, fits ? c : 0, smem, 0, 0};
@@ -514,6 +538,72 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
     return VD_ERR_CUDA;
   }
   return VD_OK;
+}
+
+// The resident kernel (vd_resident.cuh) takes an ordered eviction whose
+// clusters all run at once: it is bound by the latency of its phases, so it
+// wins where the streaming kernel has too few rows per SM to hide its own, and
+// loses once several waves of clusters follow one another (288 units of 2176
+// rows, d = 128: 167 us against 136).  C is the largest size, up to 12, that
+// leaves a CTA at least 64 rows and the launch at most two CTAs per SM, and
+// whose clusters form one wave.  Measured, streaming / resident, d = 128,
+// n = 2176: 8 units 29.0 / 19.6 us (C = 12; C = 8 20.9), 16 units 31.5 / 22.1
+// (C = 10), 32 units 35.1 / 29.3 (C = 8; C = 4 30.6); n = 1152: 96 units
+// 57.2 / 33.3 (C = 3; C = 4, 2.5 CTAs per SM, 50.3).  Both tensors get a
+// buffer where that keeps the wave (8 units 17.6 us in the kernel against
+// 20.3).  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
+// c CTAs (100 + c: with both buffers), for tests.  Returns C, or 0.
+constexpr int kResidentKind = 4;  // and 5: with the running mean
+constexpr int kResidentMinRows = 64;
+
+int resident_plan(const void* kern, long long units, int d, int capacity, bool decode,
+                  bool running, DeviceState& st, size_t* smem_out, bool* both_out) {
+  const char* env = std::getenv("VD_RESIDENT");
+  const int want = env ? std::atoi(env) : -1;
+  if (want == 0 || std::getenv("VD_CLUSTER_SIZE") || capacity > 32768) return 0;
+  if (want < 0 && units > 2LL * st.sms) return 0;
+  const int kind = kResidentKind + (running ? 1 : 0);
+  {
+    std::lock_guard<std::mutex> lk(g_mu);
+    for (int i = 0; i < st.n_choice; ++i) {
+      const ClusterChoice& e = st.choice[i];
+      if (e.kern == kern && e.units == units && e.d == d && e.capacity == capacity &&
+          e.kind == kind && e.want == want) {
+        *smem_out = e.smem;
+        *both_out = e.solo != 0;
+        return e.c;
+      }
+    }
+  }
+  auto smem_of = [&](int c, bool both) {
+    return vd::resident_layout(capacity, d, c, decode, running, both).total;
+  };
+  // units that run at once on clusters of c CTAs
+  auto at_once = [&](int c, bool both) -> long long {
+    const size_t smem = smem_of(c, both);
+    return smem > (size_t)st.smem_optin ? 0 : active_clusters(kern, units, c, smem, st);
+  };
+  int c = 0;
+  bool both = false;
+  if (want > 0) {
+    c = want % 100;
+    both = want >= 100;
+    if (c < 1 || c > vd::kResMaxCluster || at_once(c, both) < 1) c = 0;
+  } else {
+    const long long most = std::min<long long>(2LL * st.sms / units, capacity / kResidentMinRows);
+    for (c = (int)std::max(1LL, std::min(12LL, most)); c >= 1; --c)
+      if (at_once(c, false) >= units) break;
+    both = c >= 1 && at_once(c, true) >= units;
+  }
+  const size_t smem = c >= 1 ? smem_of(c, both) : 0;
+  std::lock_guard<std::mutex> lk(g_mu);
+  st.choice[st.next_choice] =
+      ClusterChoice{kern, units, d, capacity, kind, want, c, smem, both ? 1 : 0, 0};
+  st.next_choice = (st.next_choice + 1) % kChoiceSlots;
+  if (st.n_choice < kChoiceSlots) ++st.n_choice;
+  *smem_out = smem;
+  *both_out = both;
+  return c;
 }
 
 vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_variant var,
@@ -585,6 +675,25 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   a.k_new = static_cast<const uint16_t*>(k_new);
   a.v_new = static_cast<const uint16_t*>(v_new);
   a.unit_base = 0;
+  // the eviction's length update, a programmatic dependent of it
+  auto clamp_lengths = [&]() -> vd_status {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((c->n_seq + kThreads - 1) / kThreads));
+    cfg.blockDim = dim3(kThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute pdl;
+    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    pdl.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &pdl;
+    cfg.numAttrs = 1;
+    if (cudaLaunchKernelEx(&cfg, vd_len_clamp_kernel, c->len, N_dev, N, c->n_seq, c->capacity,
+                           (int)a.B, (int)a.mu_running, decode ? 1 : 0, fused ? (int)a.B : 0) !=
+        cudaSuccess) {
+      cudaGetLastError();
+      return VD_ERR_CUDA;
+    }
+    return VD_OK;
+  };
   if (use_small(c, score_only, holefill, weights, disp_out, score_k, *st)) {
     // one launch: the kernel also sets the sequences' lengths
     // grid: n_seq clusters of units_per_seq CTAs, one CTA per unit
@@ -598,6 +707,17 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   }
   size_t smem = 0;
   long long solo = 0;
+  if (!score_only && !holefill) {
+    const void* rk = resident_kernel(var, decode, fused);
+    bool both = false;
+    a.cluster = resident_plan(rk, units, c->head_dim, c->capacity, decode, mu == VD_MU_RUNNING,
+                              *st, &smem, &both);
+    if (a.cluster > 0) {
+      const vd::ResidentArgs ra{a, both ? 1 : 0};
+      r = launch(rk, units, a.cluster, smem, &ra, s, true);
+      return r != VD_OK ? r : clamp_lengths();
+    }
+  }
   a.cluster =
       cached_cluster(kern, units, c->head_dim, c->capacity, kind, holefill, *st, &smem, &solo);
   if (smem > (size_t)st->smem_optin) return VD_ERR_UNSUPPORTED;
@@ -629,23 +749,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   } else {
     r = launch(kern, units, a.cluster, smem, &a, s);
   }
-  if (r != VD_OK || score_only) return r;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((c->n_seq + kThreads - 1) / kThreads));
-  cfg.blockDim = dim3(kThreads);
-  cfg.stream = s;
-  cudaLaunchAttribute pdl;
-  pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  pdl.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &pdl;
-  cfg.numAttrs = 1;
-  if (cudaLaunchKernelEx(&cfg, vd_len_clamp_kernel, c->len, N_dev, N, c->n_seq, c->capacity,
-                         (int)a.B, (int)a.mu_running, decode ? 1 : 0, fused ? (int)a.B : 0) !=
-      cudaSuccess) {
-    cudaGetLastError();
-    return VD_ERR_CUDA;
-  }
-  return VD_OK;
+  return r != VD_OK || score_only ? r : clamp_lengths();
 }
 
 }  // namespace

@@ -299,6 +299,14 @@ __device__ __forceinline__ void cluster_arrive() {
   asm volatile("barrier.cluster.arrive.release;" ::: "memory");
 }
 
+// Arrival that orders nothing before it (the release form waits for the
+// thread's outstanding stores and copies): for barriers that only separate
+// execution, such as "every CTA has started" or "every CTA has finished
+// reading what will now be overwritten".
+__device__ __forceinline__ void cluster_arrive_relaxed() {
+  asm volatile("barrier.cluster.arrive.relaxed;" ::: "memory");
+}
+
 __device__ __forceinline__ void cluster_wait() {
   asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }

@@ -1,0 +1,204 @@
+"""The resident kernel (a unit's scored rows in the shared memory of its
+cluster) against the streaming kernel on the same inputs, over the forms it
+accepts: rules, mean modes, fused and two-call, block and decode, scoring
+options, ragged lengths and budgets, cluster sizes that divide nothing, slices
+that end mid-row-group or are empty, heavy ties and non-finite rows.
+VD_RESIDENT=0 forces the streaming kernel, VD_RESIDENT=c the resident one on
+clusters of c CTAs (100 + c: both tensors resident).  Needs a GB300.
+
+The two compute every score with the same operations in the same order; only
+the order of the mean's double-float sums differs, which moves the two-part
+mean by at most 1e-12 of the data's scale.  So scores are compared at 1e-6
+relative (16 fp32 roundings), everything else exactly, running sums at 1e-12
+of the summed magnitudes."""
+from __future__ import annotations
+
+import itertools
+
+import pytest
+import torch
+
+import paper_2609_23314_gb300 as vd
+from paper_2609_23314_gb300 import build, workloads as wl
+from vd_gpu import units_view
+
+pytestmark = pytest.mark.gpu
+
+L2, DIR, NORM = vd.VD_SCORE_L2, vd.VD_SCORE_DIR, vd.VD_SCORE_NORM
+REC, RUN = vd.VD_MU_RECOMPUTE, vd.VD_MU_RUNNING
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    vd.load_library()
+    torch.cuda.set_device(0)
+
+
+def make(n_seq, L, H, cap, d, seed, edit=None):
+    st = wl.TokenStream("gauss_outlier", n_seq * L * H, d, seed=seed)
+    k, v = st.next(cap)
+    shape = (n_seq, L, H, cap, d)
+    k, v = k.view(shape).contiguous(), v.view(shape).contiguous()
+    if edit is not None:
+        edit(k, v)
+    return k, v
+
+
+def step(force, k, v, lens, N, B, var, mu, decode, fused, budgets, options, monkeypatch):
+    """One event of the cache k, v (lens rows each, the last B of them new)
+    under VD_RESIDENT=force; every output, the cache and the status."""
+    monkeypatch.setenv("VD_RESIDENT", str(force))
+    monkeypatch.setenv("VD_SMALL_PATH", "0")
+    n_seq, L, H, cap, d = k.shape
+    us = (n_seq, L, H)
+    cache = vd.Cache(k.clone(), v.clone(), torch.tensor([n - B for n in lens], dtype=torch.int32,
+                                                        device="cuda"))
+    keys = bool(options.get("keys"))
+    rs = None
+    if mu == RUN:
+        rs = torch.zeros(us + (d,), dtype=torch.float64, device="cuda")
+        vd.vd_running_sum_init_ex(cache, keys, rs)
+    new = []
+    for t in (k, v):
+        rows = torch.stack([t[s, :, :, n - B:n] for s, n in enumerate(lens)]).contiguous()
+        new.append(rows)
+    if fused:  # the staged rows are not in the cache
+        for s, n in enumerate(lens):
+            cache.k[s, :, :, n - B:] = 0
+            cache.v[s, :, :, n - B:] = 0
+    else:
+        vd.vd_append(cache, new[0], new[1], B)
+    n_dev = torch.tensor(budgets, dtype=torch.int32, device="cuda") if budgets else None
+    kept = torch.full(us + (N,), -7, dtype=torch.int32, device="cuda")
+    ev = torch.full(us, -7, dtype=torch.int32, device="cuda")
+    sc = torch.full(us + (cap,), -3.0, device="cuda")
+    sg = torch.full(us, -3.0, device="cuda") if options.get("sigma") else None
+    attn = None
+    if options.get("attn"):
+        g = torch.Generator(device="cuda").manual_seed(3)
+        attn = torch.rand(us + (cap,), generator=g, device="cuda") * 0.02
+    if decode:
+        if fused:
+            vd.vd_append_evict_decode(cache, *new, N, n_dev, var, mu, rs, ev, kept, sc)
+        else:
+            vd.vd_evict_decode(cache, N, n_dev, var, mu, rs, ev, kept, sc)
+    elif options:
+        if fused:
+            vd.vd_append_evict_block_ex(cache, *new, B, N, n_dev, var, mu, rs, keys, attn, kept,
+                                        sc, sg)
+        else:
+            vd.vd_evict_block_ex(cache, N, n_dev, B, var, mu, rs, keys, attn, kept, sc, sg)
+    elif fused:
+        vd.vd_append_evict_block(cache, *new, B, N, n_dev, var, mu, rs, kept, sc)
+    else:
+        vd.vd_evict_block(cache, N, n_dev, B, var, mu, rs, kept, sc)
+    status = vd.vd_get_device_status()
+    return cache, rs, kept, ev, sc, sg, status
+
+
+def compare(forces, k, v, lens, N, B, var, mu, decode, fused, monkeypatch, budgets=None,
+            options=None, score_rtol=1e-6):
+    args = (k, v, lens, N, B, var, mu, decode, fused, budgets, options or {}, monkeypatch)
+    want = step(0, *args)
+    for force in forces:
+        got = step(force, *args)
+        assert got[6] == want[6]
+        assert torch.equal(got[0].len, want[0].len)
+        assert torch.equal(got[2], want[2]), force
+        assert torch.equal(got[3], want[3]), force
+        assert torch.equal(got[4] == -3.0, want[4] == -3.0)
+        torch.testing.assert_close(got[4], want[4], rtol=score_rtol, atol=0, equal_nan=True)
+        if got[5] is not None:
+            torch.testing.assert_close(got[5], want[5], rtol=1e-6, atol=0, equal_nan=True)
+        for s, n in enumerate(want[0].len.tolist()):
+            for a, b in ((got[0].k, want[0].k), (got[0].v, want[0].v)):
+                assert torch.equal(a[s, :, :, :n].view(torch.int16),
+                                   b[s, :, :, :n].view(torch.int16)), force
+        if want[1] is not None and bool(torch.isfinite(want[1]).all()):
+            scale = max(1.0, units_view(v).float().abs().nan_to_num(0, 0, 0).sum(dim=1).max().item())
+            assert torch.max(torch.abs(got[1] - want[1])).item() <= 1e-12 * scale
+
+
+FORMS = list(itertools.product([L2, DIR, NORM], [REC, RUN], [False, True], [False, True]))
+
+
+@pytest.mark.parametrize("var,mu,decode,fused", FORMS)
+def test_forms(var, mu, decode, fused, monkeypatch):
+    """Every form; ragged lengths, one sequence that does not evict; C from
+    one CTA to more CTAs than there are 4-row groups."""
+    B = 1 if decode else 37
+    for d, cap, forces in ((128, 333, (1, 3, 8, 102)), (96, 300, (2, 7, 105)), (8, 50, (1, 16, 104)),
+                           (256, 131, (4, 11))):
+        N = cap - B
+        lens = [cap, N + 1, N] if not decode else [cap, N, cap - 2]
+        lens = [max(n, B) for n in lens]
+        budgets = [N, N, N] if not decode else [N, N, N - 1]
+        k, v = make(3, 1, 2, cap, d, seed=d + B)
+        compare(forces, k, v, lens, N, B, var, mu, decode, fused, monkeypatch, budgets)
+
+
+@pytest.mark.parametrize("var,mu", [(L2, REC), (L2, RUN), (DIR, RUN), (NORM, RUN)])
+@pytest.mark.parametrize("fused", [False, True])
+@pytest.mark.parametrize("options", [dict(keys=True), dict(attn=True), dict(sigma=True),
+                                     dict(keys=True, attn=True, sigma=True)],
+                         ids=["keys", "attn", "sigma", "all"])
+def test_options(var, mu, fused, options, monkeypatch):
+    if options.get("sigma") and var != L2:
+        options = dict(options, sigma=False)
+    for d, cap, forces in ((64, 700, (1, 5, 106)), (200, 210, (3,))):
+        N, B = cap * 3 // 4, cap // 5
+        k, v = make(2, 2, 1, cap, d, seed=d)
+        compare(forces, k, v, [cap - 3, N + 2], N, B, var, mu, False, fused, monkeypatch,
+                [N, N - 5], options)
+
+
+@pytest.mark.parametrize("kind", ["all_equal", "many_equal", "two_values", "nan", "inf", "huge"])
+@pytest.mark.parametrize("decode", [False, True])
+def test_ties_and_nonfinite(kind, decode, monkeypatch):
+    """Threshold buckets with more than 256 keys, exact ties across slices,
+    keys at both ends of their range."""
+    def edit(k, v):
+        n = v.shape[3]
+        if kind == "all_equal":
+            v[:] = 1.5
+        elif kind == "many_equal":
+            v[:, :, :, n // 4:] = v[:, :, :, :1]
+        elif kind == "two_values":
+            v[:] = 1.0
+            v[:, :, :, ::3] = -1.0
+        elif kind == "nan":
+            v[:, :, :, 5, 3] = float("nan")
+        elif kind == "inf":
+            v[:, :, :, n - 1, 0] = float("inf")
+        elif kind == "huge":
+            v[:, :, :, 7] = 1e18
+            v[:, :, :, 8:40] = 0.0
+    cap = 1300
+    B = 1 if decode else 300
+    k, v = make(1, 1, 2, cap, 64, seed=9, edit=edit)
+    for var, mu in ((NORM, REC), (L2, REC)):
+        compare((1, 2, 9, 104), k, v, [cap], cap - B, B, var, mu, decode, False, monkeypatch)
+
+
+@pytest.mark.parametrize("N", [1, 2, 255, 1023])
+def test_budget_edges(N, monkeypatch):
+    cap = 1024
+    k, v = make(1, 1, 3, cap, 64, seed=N)
+    compare((1, 6, 16, 103), k, v, [cap], N, cap - N, L2, RUN, False, True, monkeypatch)
+
+
+def test_rejected_lengths_leave_the_unit_alone(monkeypatch):
+    """The same status codes as the streaming kernel, and nothing written."""
+    for force in (0, 3):
+        monkeypatch.setenv("VD_RESIDENT", str(force))
+        monkeypatch.setenv("VD_SMALL_PATH", "0")
+        for ln, n_dev, code in ((90, None, 7), (-1, None, 7), (80, 0, 8), (80, 61, 8)):
+            k, v = make(1, 1, 2, 80, 64, seed=1)
+            cache = vd.Cache(k.clone(), v.clone(), torch.tensor([ln], dtype=torch.int32,
+                                                                device="cuda"))
+            nd = None if n_dev is None else torch.tensor([n_dev], dtype=torch.int32, device="cuda")
+            vd.vd_evict_block(cache, 60, nd, 20, L2)
+            assert vd.vd_get_device_status() == code
+            assert int(cache.len[0]) == ln
+            assert torch.equal(cache.v, v) and torch.equal(cache.k, k)
