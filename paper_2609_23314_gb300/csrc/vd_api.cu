@@ -288,12 +288,36 @@ bool cluster_allowed(int c, int d) {
   return c == 1 || (total_chunks % c == 0 && total_chunks / c >= 4);
 }
 
-// CTAs per unit: C in {1, 2, 4, 8, 16}, keeping row segments of at least 64
-// bytes of [K | V].  Waves = CTAs / resident slots at that C's shared-memory
-// size.  Decode and score-only launches: the smallest C whose CTAs form one
-// nearly full wave (0.85-1) or at least two waves, so that no short tail
-// wave runs alone.  Ordered block eviction (moves most of the cache): the
-// smallest C with 0.85-1 waves or at least four, else the decode rule.
+// CTAs per unit: C in {1, 2, 4, 8}, keeping row segments of at least 64 bytes
+// of [K | V].  Waves = CTAs / resident slots at that C's shared-memory size.
+//
+// Up to about 2.6 CTAs per SM, more CTAs per unit shorten the launch (each
+// reads less, and all of them still run side by side); beyond, the CTAs of an
+// SM only share its bandwidth while every cluster barrier still costs.
+// `side` is the largest C with units * C <= 2.6 SMs that leaves a CTA at least
+// kMinRowsPerCta rows.  It is taken by ordered block eviction unless its
+// slices exceed 1.25 MB, by hole-fill decode and by score-only launches without
+// the bulk ring.  d = 128, us: ordered block, n = 1152, 96 units C = 4 39.0
+// (C = 2 42, 8 58), 192 units C = 2 55 (1 61, 4 73), 240 units C = 1 66.6
+// (2 69.5, 8 115); n = 2176, 288 units C = 1 131 (2 136); where the score pass
+// is bound by instruction issue (`heavy`: Dir, or a head dim off the batched
+// path), up to 0.95 of a wave instead (Dir, 288 units C = 2 161, C = 1 189;
+// hole-fill decode, d = 192, n = 2001, 240 units C = 2 129, C = 1 150);
+// hole-fill decode,
+// n = 4097, 192 units C = 2 50.6 (8 76), 384 units C = 1 79 (2 103); scores,
+// d = 96, n = 2048, 288 units C = 1 84 (2 90, 4 96).
+//
+// Ordered block eviction with more units, or larger slices: several waves,
+// whose tail shrinks with the slice.  The smallest C with slices of at most
+// 300 KB: 164 KB units C = 1 (800 units 102 us; C = 2 111, 4 158), 557 KB
+// units C = 2 (800 units 344; C = 1 361), prefill_wide's 2.2 MB C = 8 (568 us;
+// C = 4 586, C = 1 612).  Ordered decode, which has no select to synchronise
+// on: the largest C within 0.85 of a wave, or the smallest (up to 4) with
+// slices of at most 200 KB where that is larger (n = 4097, 128 units C = 4
+// 79.7 us, C = 2 86; 16384 units C = 4 7.28 ms, C = 1 7.37; n = 3001, 800
+// units C = 4 282 us, C = 1 313).  Hole-fill decode and score-only with more
+// units: C = 1 up to one wave, else the smallest C with two waves.
+//
 // Hole-fill block eviction (moves few rows, so the select's cluster
 // synchronisation dominates and grows with C): the smallest C with at least
 // 0.4 of a wave (one short wave beats a long tail and more cluster barriers:
@@ -303,22 +327,18 @@ bool cluster_allowed(int c, int d) {
 // least half a wave (fewer, longer contiguous slices: the prefill_wide sigma
 // pass at C=1, 0.74 waves, 0.115 ms vs C=2 0.131, C=4 0.139; 2 ring stages at
 // 3 CTAs per SM; 3 stages 0.141 ms, 4 stages 0.149).  With none such (few
-// units), the largest allowed C that
-// leaves every CTA at least kMinRowsPerCta rows of the capacity, else the
-// smallest allowed C: below that, the cluster barriers cost more than the
-// split saves.  (Measured on GB300: prefill_wide ordered C=8 (4.4 waves)
-// 0.574 ms vs C=4 (2.2) 0.586; hole-fill C=2 (1.47 waves) 0.205 vs C=4
-// 0.216; decode C=1; two units of 160 rows C=1 16.8 us vs C=4 18.5, of 600
-// rows C=4 20.9 vs C=1 26.4, of 2400 rows C=8 27.9 vs C=1 75.7.)  Where no C
-// with 64-byte segments fits the shared memory (a large capacity at a small
-// head dim), the smallest C that fits.  want
-// (VD_CLUSTER_SIZE: 1, 2, 4, 8 or 16) overrides the choice, for tuning.
+// units), the largest C that leaves every CTA at least kMinRowsPerCta rows of
+// the capacity, else the smallest allowed C.  Where no C with 64-byte segments
+// fits the shared memory (a large capacity at a small head dim), the smallest
+// C that fits.  want (VD_CLUSTER_SIZE: 1, 2, 4, 8 or 16) overrides the choice,
+// for tuning.
 constexpr int kMinRowsPerCta = 128;
 
 int choose_cluster(const void* kern, long long units, int d, int capacity, int kind,
-                   bool holefill, int want, const DeviceState& st, size_t* smem_out) {
-  const bool with_select = kind == vd::kKindBlock;
-  int chosen = 0, fallback = 0, roomy = 0, smallest = 0, narrow = 0;
+                   bool holefill, bool heavy, int want, const DeviceState& st,
+                   size_t* smem_out) {
+  int roomy = 0, smallest = 0, narrow = 0;  // see above
+  int side = 0, sliced = 0, filled = 0, waved = 0;
   for (int c = 1; c <= 16; c *= 2) {
     if (want >= 1 && c != want) continue;
     if ((d / 8 * 2) % c) continue;
@@ -330,35 +350,41 @@ int choose_cluster(const void* kern, long long units, int d, int capacity, int k
       continue;
     }
     if (occ < 1 || !cluster_fits(kern, units, c, smem, st)) continue;
-    if (want < 1 && !cluster_allowed(c, d)) {
-      // narrower row segments than preferred: only when nothing else fits
-      // (a large capacity at a small head dim)
+    if (want >= 1 || !cluster_allowed(c, d)) {
+      // forced, or narrower row segments than preferred: only when nothing
+      // else fits (a large capacity at a small head dim)
       if (narrow == 0) narrow = c;
       continue;
     }
     if (smallest == 0) smallest = c;
-    if ((capacity + c - 1) / c >= kMinRowsPerCta) roomy = c;
+    if (c > 8) continue;  // 16-CTA clusters leave SMs of a GPC idle: never the fastest
+    const long long rows = (capacity + c - 1) / c;
     const double waves = (double)(units * c) / ((double)st.sms * occ);
-    const bool full_wave = waves >= 0.85 && waves <= 1.0;
-    bool ok;
-    if (want >= 1)
-      ok = true;
-    else if (with_select && holefill)
-      ok = waves >= 0.4;
-    else if (kind == vd::kKindScoreBulk)
-      ok = waves >= 0.5;
-    else if (with_select)
-      ok = full_wave || waves >= 4.0;
-    else
-      ok = full_wave || waves >= 2.0;
-    if (ok) {
-      chosen = c;
-      break;
-    }
-    if (fallback == 0 && (full_wave || waves >= 2.0)) fallback = c;
+    const bool room = c == 1 || rows >= kMinRowsPerCta;
+    if (room) roomy = c;
+    if (room && (heavy ? waves <= 0.95 : (double)(units * c) <= 2.6 * st.sms)) side = c;
+    if (room && waves <= 0.85) filled = c;
+    if (sliced == 0 && rows * d * 2 <= (kind == vd::kKindDecode ? 200 << 10 : 300 << 10)) sliced = c;
+    const bool enough = kind == vd::kKindBlock       ? waves >= 0.4
+                        : kind == vd::kKindScoreBulk ? waves >= 0.5
+                                                     : waves <= 1.0 || waves >= 2.0;
+    if (waved == 0 && enough) waved = c;
   }
-  if (chosen == 0)
-    chosen = fallback ? fallback : roomy ? roomy : smallest ? smallest : narrow ? narrow : 1;
+  const int large = roomy ? roomy : smallest;
+  int chosen;
+  if (want >= 1 || smallest == 0) {
+    chosen = narrow ? narrow : 1;
+  } else if (kind == vd::kKindScoreBulk || (kind == vd::kKindBlock && holefill)) {
+    chosen = waved ? waved : large;
+  } else if (kind == vd::kKindBlock) {
+    const bool fits_side =
+        side && (long long)((capacity + side - 1) / side) * d * 2 <= (5LL << 20) / 4;
+    chosen = fits_side ? side : sliced ? sliced : large;
+  } else if (kind == vd::kKindDecode && !holefill) {
+    chosen = std::max(filled, std::min(sliced ? sliced : large, 4));
+  } else {
+    chosen = side ? side : waved ? waved : large;
+  }
   *smem_out = vd::smem_layout(capacity, chosen, kind).total;
   return chosen;
 }
@@ -418,7 +444,7 @@ long long split_plan(const void* kern, long long units, int d, int capacity, int
 // VD_SOLO_UNITS with it forces a split whose first launch runs that many
 // units (at most all but one) one CTA each, for tests.
 int cached_cluster(const void* kern, long long units, int d, int capacity, int kind,
-                   bool holefill, DeviceState& st, size_t* smem_out, long long* solo_out) {
+                   bool holefill, bool heavy, DeviceState& st, size_t* smem_out, long long* solo_out) {
   const char* env = std::getenv("VD_CLUSTER_SIZE");
   const int want = env ? std::atoi(env) : 0;
   // want_solo: the forced first part (VD_SOLO_UNITS, with a forced cluster
@@ -443,7 +469,7 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
       }
     }
   }
-  int c = choose_cluster(kern, units, d, capacity, kind, holefill, want, st, smem_out);
+  int c = choose_cluster(kern, units, d, capacity, kind, holefill, heavy, want, st, smem_out);
   long long solo = 0;
   if (want >= 1 && want_solo > 0) {
     solo = std::min(want_solo, units - 1);
@@ -719,7 +745,8 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     }
   }
   a.cluster =
-      cached_cluster(kern, units, c->head_dim, c->capacity, kind, holefill, *st, &smem, &solo);
+      cached_cluster(kern, units, c->head_dim, c->capacity, kind, holefill,
+                     !vd::score_bulk((int)var, c->head_dim), *st, &smem, &solo);
   if (smem > (size_t)st->smem_optin) return VD_ERR_UNSUPPORTED;
 
   if (solo > 0) {
