@@ -19,18 +19,18 @@
 #include "vd_small.cuh"
 
 namespace vd {
-const void* evict_kernel_l2(bool decode, bool holefill, bool fused);
+const void* evict_kernel_l2(bool decode, bool holefill, bool fused, bool general);
 const void* evict_kernel_dir(bool decode, bool holefill, bool fused);
-const void* evict_kernel_norm(bool decode, bool holefill, bool fused);
+const void* evict_kernel_norm(bool decode, bool holefill, bool fused, bool general);
 const void* small_kernel_l2(bool decode, bool fused);
 const void* small_kernel_dir(bool decode, bool fused);
 const void* small_kernel_norm(bool decode, bool fused);
 const void* resident_kernel_l2(bool decode, bool fused);
 const void* resident_kernel_dir(bool decode, bool fused);
 const void* resident_kernel_norm(bool decode, bool fused);
-const void* score_kernel_l2();
+const void* score_kernel_l2(bool general);
 const void* score_kernel_dir();
-const void* score_kernel_norm();
+const void* score_kernel_norm(bool general);
 }  // namespace vd
 
 using vd::kThreads;
@@ -146,19 +146,21 @@ constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 DeviceState g_dev[kMaxDevices];
 
-const void* evict_kernel(vd_variant var, bool decode, bool holefill, bool fused) {
+// general: the score pass for any rule and head dim, else the batched one
+// (vd::batched_scores)
+const void* evict_kernel(vd_variant var, bool decode, bool holefill, bool fused, bool general) {
   switch (var) {
-    case VD_SCORE_L2: return vd::evict_kernel_l2(decode, holefill, fused);
+    case VD_SCORE_L2: return vd::evict_kernel_l2(decode, holefill, fused, general);
     case VD_SCORE_DIR: return vd::evict_kernel_dir(decode, holefill, fused);
-    default: return vd::evict_kernel_norm(decode, holefill, fused);
+    default: return vd::evict_kernel_norm(decode, holefill, fused, general);
   }
 }
 
-const void* score_kernel(vd_variant var) {
+const void* score_kernel(vd_variant var, bool general) {
   switch (var) {
-    case VD_SCORE_L2: return vd::score_kernel_l2();
+    case VD_SCORE_L2: return vd::score_kernel_l2(general);
     case VD_SCORE_DIR: return vd::score_kernel_dir();
-    default: return vd::score_kernel_norm();
+    default: return vd::score_kernel_norm(general);
   }
 }
 
@@ -203,9 +205,9 @@ vd_status device_state(DeviceState** out) {
                              st.smem_optin) != cudaSuccess)
       return VD_ERR_CUDA;
     for (int var = 0; var < 3; ++var)
-      for (int kind = 0; kind < 8; ++kind) {
-        const void* kern =
-            evict_kernel((vd_variant)var, (kind & 1) != 0, (kind & 2) != 0, (kind & 4) != 0);
+      for (int kind = 0; kind < 16; ++kind) {
+        const void* kern = evict_kernel((vd_variant)var, (kind & 1) != 0, (kind & 2) != 0,
+                                        (kind & 4) != 0, (kind & 8) != 0);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  st.smem_optin) != cudaSuccess ||
             cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
@@ -213,9 +215,9 @@ vd_status device_state(DeviceState** out) {
           return VD_ERR_CUDA;
       }
     for (int var = 0; var < 3; ++var)
-      for (int kind = 0; kind < 9; ++kind) {
+      for (int kind = 0; kind < 10; ++kind) {
         const bool dec = (kind & 1) != 0, fus = (kind & 2) != 0;
-        const void* kern = kind == 8  ? score_kernel((vd_variant)var)
+        const void* kern = kind >= 8  ? score_kernel((vd_variant)var, kind == 9)
                            : kind < 4 ? small_kernel((vd_variant)var, dec, fus)
                                       : resident_kernel((vd_variant)var, dec, fus);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -296,7 +298,8 @@ bool cluster_allowed(int c, int d) {
 // SM only share its bandwidth while every cluster barrier still costs.
 // `side` is the largest C with units * C <= 2.6 SMs that leaves a CTA at least
 // kMinRowsPerCta rows.  It is taken by ordered block eviction unless its
-// slices exceed 1.25 MB, by hole-fill decode and by score-only launches without
+// slices exceed 1.25 MB (300 KB where the mean is recomputed, `resum`: 288
+// units of 2176 rows C = 2 146 us, C = 1 156), by hole-fill decode and by score-only launches without
 // the bulk ring.  d = 128, us: ordered block, n = 1152, 96 units C = 4 39.0
 // (C = 2 42, 8 58), 192 units C = 2 55 (1 61, 4 73), 240 units C = 1 66.6
 // (2 69.5, 8 115); n = 2176, 288 units C = 1 131 (2 136); where the score pass
@@ -335,7 +338,7 @@ bool cluster_allowed(int c, int d) {
 constexpr int kMinRowsPerCta = 128;
 
 int choose_cluster(const void* kern, long long units, int d, int capacity, int kind,
-                   bool holefill, bool heavy, int want, const DeviceState& st,
+                   bool holefill, bool heavy, bool resum, int want, const DeviceState& st,
                    size_t* smem_out) {
   int roomy = 0, smallest = 0, narrow = 0;  // see above
   int side = 0, sliced = 0, filled = 0, waved = 0;
@@ -378,7 +381,8 @@ int choose_cluster(const void* kern, long long units, int d, int capacity, int k
     chosen = waved ? waved : large;
   } else if (kind == vd::kKindBlock) {
     const bool fits_side =
-        side && (long long)((capacity + side - 1) / side) * d * 2 <= (5LL << 20) / 4;
+        side && (long long)((capacity + side - 1) / side) * d * 2 <=
+                    (resum ? 300 << 10 : (5LL << 20) / 4);
     chosen = fits_side ? side : sliced ? sliced : large;
   } else if (kind == vd::kKindDecode && !holefill) {
     chosen = std::max(filled, std::min(sliced ? sliced : large, 4));
@@ -444,7 +448,8 @@ long long split_plan(const void* kern, long long units, int d, int capacity, int
 // VD_SOLO_UNITS with it forces a split whose first launch runs that many
 // units (at most all but one) one CTA each, for tests.
 int cached_cluster(const void* kern, long long units, int d, int capacity, int kind,
-                   bool holefill, bool heavy, DeviceState& st, size_t* smem_out, long long* solo_out) {
+                   bool holefill, bool heavy, bool resum, DeviceState& st, size_t* smem_out, long long* solo_out) {
+  const int key = kind | (resum ? 256 : 0);  // of the remembered choice
   const char* env = std::getenv("VD_CLUSTER_SIZE");
   const int want = env ? std::atoi(env) : 0;
   // want_solo: the forced first part (VD_SOLO_UNITS, with a forced cluster
@@ -462,14 +467,14 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
     for (int i = 0; i < st.n_choice; ++i) {
       const ClusterChoice& e = st.choice[i];
       if (e.kern == kern && e.units == units && e.d == d && e.capacity == capacity &&
-          e.kind == kind && e.want == want && e.want_solo == want_solo) {
+          e.kind == key && e.want == want && e.want_solo == want_solo) {
         *smem_out = e.smem;
         *solo_out = e.solo;
         return e.c;
       }
     }
   }
-  int c = choose_cluster(kern, units, d, capacity, kind, holefill, heavy, want, st, smem_out);
+  int c = choose_cluster(kern, units, d, capacity, kind, holefill, heavy, resum, want, st, smem_out);
   long long solo = 0;
   if (want >= 1 && want_solo > 0) {
     solo = std::min(want_solo, units - 1);
@@ -486,7 +491,7 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
   }
   std::lock_guard<std::mutex> lk(g_mu);
   st.choice[st.next_choice] =
-      ClusterChoice{kern, units, d, capacity, kind, want, c, *smem_out, solo, want_solo};
+      ClusterChoice{kern, units, d, capacity, key, want, c, *smem_out, solo, want_solo};
   st.next_choice = (st.next_choice + 1) % kChoiceSlots;
   if (st.n_choice < kChoiceSlots) ++st.n_choice;
   *solo_out = solo;
@@ -664,14 +669,15 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   if (r != VD_OK) return r;
 
   // score-only launches have their own instantiation (no per-token buffers)
-  const int kind = score_only ? (vd::score_bulk((int)var, c->head_dim) ? vd::kKindScoreBulk
-                                                                       : vd::kKindScore)
+  const bool general = !vd::batched_scores((int)var, c->head_dim);
+  const int kind = score_only ? (general ? vd::kKindScore : vd::kKindScoreBulk)
                  : decode     ? vd::kKindDecode
                               : vd::kKindBlock;
   if (kind == vd::kKindBlock && c->capacity > 65536) return VD_ERR_UNSUPPORTED;  // 16-bit lists
   if (vd::smem_layout(c->capacity, 16, kind).total > (size_t)st->smem_optin)
     return VD_ERR_UNSUPPORTED;
-  const void* kern = score_only ? score_kernel(var) : evict_kernel(var, decode, holefill, fused);
+  const void* kern = score_only ? score_kernel(var, general)
+                                : evict_kernel(var, decode, holefill, fused, general);
   const long long units = (long long)c->n_seq * c->n_layer * c->n_kv_head;
 
   vd::EvictArgs a;
@@ -745,8 +751,8 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     }
   }
   a.cluster =
-      cached_cluster(kern, units, c->head_dim, c->capacity, kind, holefill,
-                     !vd::score_bulk((int)var, c->head_dim), *st, &smem, &solo);
+      cached_cluster(kern, units, c->head_dim, c->capacity, kind, holefill, general,
+                     mu == VD_MU_RECOMPUTE && var != VD_SCORE_NORM, *st, &smem, &solo);
   if (smem > (size_t)st->smem_optin) return VD_ERR_UNSUPPORTED;
 
   if (solo > 0) {

@@ -133,6 +133,12 @@ __device__ __forceinline__ unsigned long long ld_shared_b64(uint32_t addr) {
   return r;
 }
 
+// Two of them from one 16-byte vector (volatile, for the same reason).
+__device__ __forceinline__ void ld_shared_2b64(uint32_t addr, unsigned long long& a,
+                                               unsigned long long& b) {
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr));
+}
+
 __device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z),
                "r"(v.w)

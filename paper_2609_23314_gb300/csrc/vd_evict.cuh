@@ -57,6 +57,7 @@
 #pragma once
 
 #include <climits>
+#include <cstddef>
 #include <cstdint>
 #include <type_traits>
 
@@ -95,6 +96,11 @@ namespace vd {
 #endif
 #ifndef VD_DECODE_MIN_CTAS
 #define VD_DECODE_MIN_CTAS 4
+#endif
+// Kernels with the general score pass: its batch of rows needs the registers
+// of 3 (at 4 CTAs per SM, 64 registers, it spilled).
+#ifndef VD_GENERAL_MIN_CTAS
+#define VD_GENERAL_MIN_CTAS 3
 #endif
 // Score-only launches (vd_score, vd_score_ex) have their own instantiation:
 // no select, slot lists or compaction, so a deeper ring fits at a lower
@@ -136,9 +142,10 @@ __host__ __device__ constexpr int ring_bytes(int kind) {
                                    : DecodeRing::kBytes;
 }
 
-// Whether a score-only launch takes the bulk ring: the batched L2 / Norm
-// score pass, whose stage of 32 KB is exactly one batch of rows per lane group.
-__host__ __device__ constexpr bool score_bulk(int var, int d) {
+// The batched score passes: L2 and Norm at head dims with one 16-byte chunk
+// per lane (score-only launches: a bulk-ring stage of 32 KB is then exactly one
+// batch of rows per lane group).  Everything else takes score_rows_general.
+__host__ __device__ constexpr bool batched_scores(int var, int d) {
   return var != 1 && (d == 64 || d == 128 || d == 256);
 }
 
@@ -186,11 +193,12 @@ struct Smem {
   float mu[256];    // the mean rounded to fp32 ...
   float mulo[256];  // ... and its remainder (mean = mu + mulo to ~2^-44 relative),
                     // pair-transposed: column c at lo_index(c, d / 8)
+  uint32_t ghist[256];  // (the general score pass keeps the remainder twice per
+                        // column, over mulo and ghist: dup_index)
   float acc_hi[256];  // this CTA's partial column sums (read by peer CTAs)
   float acc_lo[256];
   double snew[256];       // running mode: the running sum plus the appended rows
   uint32_t hist[2][256];  // this CTA's radix histograms (read by peers)
-  uint32_t ghist[256];
   int scan[kWarps];
   float fsh[kWarps];
   unsigned long long best;  // decode: this CTA's (key, -tie-break) minimum
@@ -216,6 +224,14 @@ __host__ __device__ constexpr size_t align16(size_t x) { return (x + 15) & ~(siz
 // pair k of chunk ci at floats 2 * (k * d8 + ci) and + 1.
 __device__ __forceinline__ int lo_index(int c, int d8) {
   return 2 * (((c & 7) >> 1) * d8 + (c >> 3)) + (c & 1);
+}
+
+// General score pass: column c's remainder is the pair of floats (x, x) at this
+// entry of the 2 KB over Smem::mulo and Smem::ghist.  Columns 2p and 2p + 1 of a
+// chunk are one 16-byte vector, 512 bytes from the next p's: a warp's loads
+// hit distinct banks at constant offsets.
+__device__ __forceinline__ int dup_index(int c) {
+  return ((c & 7) >> 1) * 64 + (c >> 3) * 2 + (c & 1);
 }
 
 // Byte offsets of the variable parts; the host sizes the launch with the same
@@ -374,9 +390,12 @@ __device__ __forceinline__ void score_rows_fast(const uint16_t* __restrict__ row
       cp_async_wait<kStages - 1>();
 #pragma unroll
       for (int u = 0; u < kItems; ++u) {
-        const int k = st * kItems + u;
+        // a row past the end shares no sum with another: its slot may hold
+        // anything (the decode kernels' batches of 4 test it all the same:
+        // without the test they spill)
         uint4 q = make_uint4(0u, 0u, 0u, 0u);
-        if (g + k * kGroups < R) q = ld_shared16(slot(st % kStages, u));
+        if (kBatch == 8 || g + (st * kItems + u) * kGroups < R)
+          q = ld_shared16(slot(st % kStages, u));
         part[sb * kItems + u] = chunk_sq<VAR, LPR>(q, m2, lo_addr);
       }
       issue(st + kStages);
@@ -398,6 +417,157 @@ __device__ __forceinline__ void score_rows_fast(const uint16_t* __restrict__ row
     if (ci % kSpread == 0) {
       const int j = g + (b * kBatch + ci / kSpread) * kGroups;
       if (j < R) finish(R - 1 - j, sqrtf(part[0]));
+    }
+  }
+  cp_async_wait<0>();
+}
+
+// Score pass over R contiguous rows for the head dims score_rows_fast does not
+// take, and for the Dir rule: lpr lanes per row (the next power of two >= d / 8;
+// idle lanes hold zeros), rows visited from the last to the first.  Rows stream
+// through the thread-private ring.  The two rows of a stage go through packed
+// fp32 pairs, one row per half: per row the scalar operations in their order,
+// half the instructions.  A batch of rows (4; 2 for Dir, whose second sum needs
+// the first one's result) is reduced by one transposed butterfly at lane
+// distance 1, 2, 4, ..., which hands each of the batch's first lanes one row
+// to finish.  Bound by instruction issue (133 warp instructions per row before
+// the pairs, at d = 192).  us, row by row / batched / in pairs too: hole-fill
+// block, 480 units of 2128 rows, d = 192 345 / 177 / 154, d = 96 181 / 101 /
+// 91; hole-fill decode d = 192 236 / 163 / 109; Dir, 288 units of 2176
+// rows, d = 128 161 / 157 / 153.
+template <int VAR, class Ring, int BATCH, class Finish>
+__device__ __forceinline__ void score_rows_general(const uint16_t* rows, int d, int lpr, int R,
+                                                   const Smem& S, Finish finish, uint32_t ring) {
+  constexpr int kStages = Ring::kStages, kItems = Ring::kItems;
+  constexpr int kBatch = BATCH, kLog = BATCH == 4 ? 2 : 1;
+  static_assert((1 << kLog) == kBatch && kItems == 2, "a stage is one pair of rows");
+  static_assert(VAR != 1 || kBatch == 2, "Dir: two squared norms per batch");
+  const int tid = threadIdx.x, lane = tid & 31, d8 = d >> 3;
+  const int ci = lane & (lpr - 1), g = tid / lpr, ng = kThreads / lpr;
+  const bool active = ci < d8;
+  unsigned long long mm[8];  // this lane's columns of the mean's fp32 part, in both halves
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const float m = (VAR != 2 && active) ? S.mu[ci * 8 + k] : 0.f;
+    mm[k] = f2_pack(m, m);
+  }
+  // ... and of its remainder, read at each use (see chunk_sq)
+  const uint32_t lo_addr = smem_addr(S.mulo) + (uint32_t)ci * 16u;
+  const bool mu_zero = VAR == 1 && S.mu_zero;
+  const float inv_mnorm = VAR == 1 ? S.inv_mnorm : 0.f;
+  const int nst = (R + ng * kItems - 1) / (ng * kItems);
+  // the next row this thread copies, and its visit (row R - 1 - next_i)
+  const uint16_t* next = rows + (size_t)(R - 1) * d + ci * 8 - (size_t)g * d;
+  int next_i = active ? g : R;
+  const int hop = ng * d;
+  const uint32_t my = ring + (uint32_t)tid * 16u;
+  auto slot = [&](int s, int u) { return my + (uint32_t)((s * kItems + u) * kThreads * 16); };
+  auto issue = [&](int st) {
+#pragma unroll
+    for (int u = 0; u < kItems; ++u) {
+      if (next_i < R) cp_async16(slot(st % kStages, u), next);
+      next -= hop;
+      next_i += ng;
+    }
+    cp_async_commit();
+  };
+  for (int st = 0; st < kStages; ++st) issue(st);
+  const int nbatch = (nst + kBatch / kItems - 1) / (kBatch / kItems);
+  for (int b = 0; b < nbatch; ++b) {
+    float part[kBatch], nv[2];
+#pragma unroll
+    for (int sb = 0; sb < kBatch / kItems; ++sb) {
+      const int st = b * (kBatch / kItems) + sb;
+      cp_async_wait<kStages - 1>();
+      // The stage's two rows.  Slots of idle lanes and of rows past the end
+      // hold anything: idle lanes' sums are dropped below, and a row past the
+      // end shares no sum with another.
+      uint32_t wa[4], wb[4];
+      {
+        const uint4 q = ld_shared16(slot(st % kStages, 0)), r = ld_shared16(slot(st % kStages, 1));
+        wa[0] = q.x, wa[1] = q.y, wa[2] = q.z, wa[3] = q.w;
+        wb[0] = r.x, wb[1] = r.y, wb[2] = r.z, wb[3] = r.w;
+      }
+      issue(st + kStages);
+      auto even = [&](int k) {
+        return f2_pack(__uint_as_float(wa[k] << 16), __uint_as_float(wb[k] << 16));
+      };
+      auto odd = [&](int k) {
+        return f2_pack(__uint_as_float(wa[k] & 0xffff0000u), __uint_as_float(wb[k] & 0xffff0000u));
+      };
+      unsigned long long lam = 0ull;  // Dir: -|v| / |mean| of both rows
+      if (VAR == 1) {
+        unsigned long long n2 = 0ull;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          const unsigned long long x0 = even(k), x1 = odd(k);
+          n2 = f2_fma(x0, x0, n2);
+          n2 = f2_fma(x1, x1, n2);
+        }
+        f2_unpack(n2, nv[0], nv[1]);
+        if (!active) nv[0] = nv[1] = 0.f;
+        for (int off = 1; off < lpr; off <<= 1) {
+#pragma unroll
+          for (int u = 0; u < 2; ++u) nv[u] += __shfl_xor_sync(kFull, nv[u], off);
+        }
+        lam = f2_pack(-(sqrtf(nv[0]) * inv_mnorm), -(sqrtf(nv[1]) * inv_mnorm));
+      }
+      unsigned long long acc = 0ull;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        unsigned long long x0 = even(k), x1 = odd(k);
+        if (VAR != 2) {
+          unsigned long long l0, l1;
+          ld_shared_2b64(lo_addr + (uint32_t)(k * 512), l0, l1);
+          // Dir: 1 - cos(v, m) = |w|^2 / (2 |v|^2) with w = v - (|v| / |m|) m:
+          // each w_c is one fused multiply-add of the row and the
+          // double-float mean, rounded relative to w_c itself, so the
+          // score's error stays relative to the score even where v and m
+          // are nearly parallel (1 - cos computed directly would cancel)
+          x0 = VAR == 0 ? f2_sub(f2_sub(x0, mm[2 * k]), l0)
+                        : f2_fma(lam, l0, f2_fma(lam, mm[2 * k], x0));
+          x1 = VAR == 0 ? f2_sub(f2_sub(x1, mm[2 * k + 1]), l1)
+                        : f2_fma(lam, l1, f2_fma(lam, mm[2 * k + 1], x1));
+        }
+        acc = f2_fma(x0, x0, acc);
+        acc = f2_fma(x1, x1, acc);
+      }
+      float a0, a1;
+      f2_unpack(acc, a0, a1);
+      part[sb * 2] = active ? a0 : 0.f;
+      part[sb * 2 + 1] = active ? a1 : 0.f;
+    }
+    auto value = [&](float t, float v2) {
+      return VAR == 1 ? ((v2 > 0.f && !mu_zero) ? (0.5f * t) / v2 : 1.f) : sqrtf(t);
+    };
+    if (lpr >= kBatch) {
+      const float nk = VAR == 1 ? ((ci & 1) ? nv[1] : nv[0]) : 0.f;  // of this lane's row
+#pragma unroll
+      for (int s = 0; s < kLog; ++s) {
+        const int h = kBatch >> (s + 1), off = 1 << s;
+        const bool upper = (ci & off) != 0;
+#pragma unroll
+        for (int k = 0; k < h; ++k) {
+          const float send = upper ? part[k] : part[k + h];
+          const float keep = upper ? part[k + h] : part[k];
+          part[k] = keep + __shfl_xor_sync(kFull, send, off);
+        }
+      }
+      for (int off = kBatch; off < lpr; off <<= 1)
+        part[0] += __shfl_xor_sync(kFull, part[0], off);
+      const int r = kBatch == 2 ? ci : 2 * (ci & 1) + ((ci >> 1) & 1);
+      const int i = g + (b * kBatch + r) * ng;
+      if (ci < kBatch && i < R) finish(R - 1 - i, value(part[0], nk));
+    } else {
+      for (int off = 1; off < lpr; off <<= 1) {
+#pragma unroll
+        for (int k = 0; k < kBatch; ++k) part[k] += __shfl_xor_sync(kFull, part[k], off);
+      }
+#pragma unroll
+      for (int k = 0; k < kBatch; ++k) {
+        const int i = g + (b * kBatch + k) * ng;
+        if (ci == 0 && i < R) finish(R - 1 - i, value(part[k], VAR == 1 ? nv[k & 1] : 0.f));
+      }
     }
   }
   cp_async_wait<0>();
@@ -485,6 +655,7 @@ __device__ __forceinline__ void sum_rows(int chunk0, int nchunks, int P, int cou
   merge_columns(hi, lo, P, active, (chunk0 + ci) * 8, S.acc_hi, S.acc_lo);
 }
 
+static_assert(offsetof(Smem, ghist) == offsetof(Smem, mulo) + 1024, "dup_index");
 static_assert(kBulkStages >= 2 && kBulkStages <= 4, "bulk ring: 2 to 4 stages (Smem::bar)");
 
 // A ring of bulk copies over this CTA's ring region: kBulkStages slots of
@@ -608,10 +779,10 @@ __device__ __forceinline__ void score_rows_bulk(BulkRing& br, const uint16_t* ro
         float part[kBatch];
 #pragma unroll
         for (int k = 0; k < kBatch; ++k) {
+          // (a row past the end shares no sum with another: its bytes may be anything)
           const int r = g + k * kGroups;
-          uint4 q = make_uint4(0u, 0u, 0u, 0u);
-          if (r < cnt) q = ld_shared16(st + (uint32_t)(r * kRowBytes + ci * 16));
-          part[k] = chunk_sq<VAR, LPR>(q, m2, lo_addr);
+          part[k] = chunk_sq<VAR, LPR>(ld_shared16(st + (uint32_t)(r * kRowBytes + ci * 16)), m2,
+                                       lo_addr);
         }
 #pragma unroll
         for (int j = 0; j < 3; ++j) {
@@ -1261,10 +1432,13 @@ __device__ __forceinline__ void move_rows_retire(uint16_t* kb, uint16_t* vb, int
 // caller's staging buffers (vd_append_evict_*); the other kernels carry none
 // of that code.  SCORE: the score-only launches (vd_score, vd_score_ex:
 // mean, scores and sigma, nothing evicted), instantiated with DECODE set
-// and their own ring and occupancy.
-template <int VAR, bool DECODE, bool HF, bool FUSED, bool SCORE>
+// and their own ring and occupancy.  GEN: the score pass for any head dim and
+// rule (score_rows_general); without it, d is 64, 128 or 256 and the rule L2
+// or Norm (batched_scores), so neither carries the other's code.
+template <int VAR, bool DECODE, bool HF, bool FUSED, bool SCORE, bool GEN>
 __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
   static_assert(!SCORE || (DECODE && !HF && !FUSED), "score-only instantiation");
+  static_assert(GEN || VAR != 1, "Dir scores on the general path");
   extern __shared__ __align__(16) unsigned char smem_raw[];
   Smem& S = *reinterpret_cast<Smem*>(smem_raw);
   using Ring = RingShape<SCORE ? ScoreRing::kStages : DECODE ? DecodeRing::kStages
@@ -1274,7 +1448,7 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
   constexpr bool score_only = SCORE;
   const int C = a.cluster;
   // score-only at head dims 64, 128, 256 (L2, Norm): the bulk-copy ring
-  const bool bulk = SCORE && score_bulk(VAR, a.d);
+  constexpr bool bulk = SCORE && !GEN;
   const int kind = SCORE ? (bulk ? kKindScoreBulk : kKindScore) : DECODE ? kKindDecode : kKindBlock;
   const SmemLayout L = smem_layout(a.capacity, C, kind);
   const uint32_t ring = smem_addr(smem_raw + L.ring);
@@ -1329,9 +1503,7 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
   }
   if (score_only && n == 0) return;
   BulkRing br{0u, 0u, 0};
-  if constexpr (SCORE) {
-    if (bulk) br = bulk_ring_init(ring, S);
-  }
+  if constexpr (bulk) br = bulk_ring_init(ring, S);
 
   // column slice of [K | V] this CTA compacts; the running sum is kept for
   // the part of it that lies in the scored tensor (V, or K for the key-side
@@ -1401,14 +1573,9 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
     // the running sum is loaded before the row sum, whose latency hides it
     const double rs_own = run && tid < d ? a.running_sum[(size_t)u * d + tid] : 0.0;
     const uint16_t* pb = srange(p0, cnt);  // nullptr only where the range straddles
-    bool summed = false;
-    if constexpr (SCORE) {
-      if (bulk) {  // score-only rows are never staged: one contiguous range
-        sum_rows_bulk(br, pb, cnt, d, lpr, S, a.status);
-        summed = true;
-      }
-    }
-    if (!summed)
+    if constexpr (bulk)  // score-only rows are never staged: one contiguous range
+      sum_rows_bulk(br, pb, cnt, d, lpr, S, a.status);
+    else
       sum_rows<Ring, kPackedSum>(0, d8, lpr, cnt,
                      [&](int i) -> const uint16_t* {
                        if constexpr (FUSED) return pb ? pb + (size_t)i * d : srow(p0 + i);
@@ -1436,7 +1603,11 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
       const double m = sum / (double)n;
       const float mh = (float)m;
       S.mu[tid] = mh;
-      S.mulo[lo_index(tid, d8)] = (float)(m - (double)mh);
+      const float ml = (float)(m - (double)mh);
+      if constexpr (GEN)
+        reinterpret_cast<float2*>(S.mulo)[dup_index(tid)] = make_float2(ml, ml);
+      else
+        S.mulo[lo_index(tid, d8)] = ml;
     }
     __syncthreads();
     if (VAR == 1) {
@@ -1463,21 +1634,6 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
   // sigma of the L2 scores (host-checked; compiled into the L2 kernels only)
   const bool disp = VAR == 0 && a.disp_out != nullptr;
   {
-    const int ci = lane & (lpr - 1);
-    const bool active = ci < d8;
-    float m8[8];  // this lane's columns of the mean (fp32 part)
-#pragma unroll
-    for (int k = 0; k < 8; ++k) m8[k] = (VAR != 2 && active) ? S.mu[ci * 8 + k] : 0.f;
-    // ... and of its remainder, read in pairs at each use (see chunk_sq)
-    const uint32_t lo_addr = smem_addr(S.mulo) + (uint32_t)(active ? ci : 0) * 8u;
-    auto lo_pair = [&](int k, float& l0, float& l1) {
-      const unsigned long long p = ld_shared_b64(lo_addr + (uint32_t)(k * d8 * 8));
-      l0 = __uint_as_float((uint32_t)p);
-      l1 = __uint_as_float((uint32_t)(p >> 32));
-      if (!active) l0 = l1 = 0.f;
-    };
-    const bool mu_zero = VAR == 1 && S.mu_zero;
-    const float inv_mnorm = VAR == 1 ? S.inv_mnorm : 0.f;
     const bool weighted = !DECODE && a.weights != nullptr;
     float ds_hi = 0.f, ds_lo = 0.f, dq_hi = 0.f, dq_lo = 0.f;  // dispersion sums
     unsigned long long best = ~0ull;  // (key, tie-break) of this thread's minimum
@@ -1516,22 +1672,19 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
         }
       }
     };
-    bool fast = false;
     // rows per batch: 4 in the ordered decode kernels, whose other live state
     // (the running arg-min, the staged-row pointers) leaves no room for 8
     // rows' partial sums within 64 registers without spilling
-    constexpr int kScoreBatch = DECODE && !HF ? 4 : 8;
-    if constexpr (VAR != 1) {  // head dims 64, 128, 256: one 16-byte chunk per lane
+    constexpr int kScoreBatch = DECODE ? 4 : 8;
+    if constexpr (!GEN) {  // head dims 64, 128, 256: one 16-byte chunk per lane
       // cache rows [r0, c_end), then (fused append) staging rows [c_end, r1)
       const int c_end = min(r1, max(r0, first_stage));
       auto run = [&](auto lanes) {
         constexpr int LPR = decltype(lanes)::value;
-        if constexpr (SCORE) {
-          if (bulk) {
-            score_rows_bulk<VAR, LPR>(br, sb + (size_t)r0 * d, r1 - r0, S.mu, S.mulo, finish_row,
-                                      a.status);
-            return;
-          }
+        if constexpr (bulk) {
+          score_rows_bulk<VAR, LPR>(br, sb + (size_t)r0 * d, r1 - r0, S.mu, S.mulo, finish_row,
+                                    a.status);
+          return;
         }
         if (r1 > c_end)
           score_rows_fast<VAR, LPR, Ring, kScoreBatch>(
@@ -1541,70 +1694,20 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
           score_rows_fast<VAR, LPR, Ring, kScoreBatch>(sb + (size_t)r0 * d, c_end - r0, S.mu,
                                                        S.mulo, finish_row, ring);
       };
-      fast = true;
       if (d == 128) run(std::integral_constant<int, 16>{});
       else if (d == 256) run(std::integral_constant<int, 32>{});
-      else if (d == 64) run(std::integral_constant<int, 8>{});
-      else fast = false;
+      else run(std::integral_constant<int, 8>{});
+    } else {
+      const int c_end = min(r1, max(r0, first_stage));
+#pragma unroll 1
+      for (int part = FUSED ? 1 : 0; part >= 0; --part) {  // staged rows, then cache rows
+        const int x = part ? c_end : r0, y = part ? r1 : c_end;
+        if (x < y)
+          score_rows_general<VAR, Ring, VAR == 1 || (DECODE && !HF && FUSED) ? 2 : 4>(
+              part ? snu + (size_t)(x - first_stage) * d : sb + (size_t)x * d, d, lpr, y - x, S,
+              [&](int j, float sc) { finish_row(x - r0 + j, sc); }, ring);
+      }
     }
-    const uint16_t* rb = srange(r0, r1 - r0);  // nullptr only where the range straddles
-    const int nr = r1 - r0;  // rows visited last to first, as in score_rows_fast
-    if (!fast) stream_rows<Ring>(
-        0, d8, lpr, nr,
-        [&](int i) -> const uint16_t* {
-          if constexpr (FUSED) return rb ? rb + (size_t)(nr - 1 - i) * d : srow(r1 - 1 - i);
-          else return rb + (size_t)(nr - 1 - i) * d;
-        },
-        [&](int item, bool in, const uint4& q) {
-          float x[8];
-          unpack8(q, x);
-          float s;
-          if (VAR == 0) {
-            float acc = 0.f;
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-              float l0, l1;
-              lo_pair(k >> 1, l0, l1);
-              const float dv0 = (x[k] - m8[k]) - l0;
-              const float dv1 = (x[k + 1] - m8[k + 1]) - l1;
-              acc = fmaf(dv0, dv0, acc);
-              acc = fmaf(dv1, dv1, acc);
-            }
-            for (int off = 1; off < lpr; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
-            s = sqrtf(acc);
-          } else if (VAR == 2) {
-            float acc = 0.f;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) acc = fmaf(x[k], x[k], acc);
-            for (int off = 1; off < lpr; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
-            s = sqrtf(acc);
-          } else {
-            // 1 - cos(v, m) = |w|^2 / (2 |v|^2) with w = v - (|v| / |m|) m:
-            // each w_c is one fused multiply-add of the row and the
-            // double-float mean, rounded relative to w_c itself, so the
-            // score's error stays relative to the score even where v and m
-            // are nearly parallel (1 - cos computed directly would cancel)
-            float nv = 0.f;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) nv = fmaf(x[k], x[k], nv);
-            for (int off = 1; off < lpr; off <<= 1) nv += __shfl_xor_sync(kFull, nv, off);
-            const float lam = sqrtf(nv) * inv_mnorm;
-            float acc = 0.f;
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-              float l0, l1;
-              lo_pair(k >> 1, l0, l1);
-              const float w0 = fmaf(-lam, l0, fmaf(-lam, m8[k], x[k]));
-              const float w1 = fmaf(-lam, l1, fmaf(-lam, m8[k + 1], x[k + 1]));
-              acc = fmaf(w0, w0, acc);
-              acc = fmaf(w1, w1, acc);
-            }
-            for (int off = 1; off < lpr; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
-            s = (nv > 0.f && !mu_zero) ? (0.5f * acc) / nv : 1.f;
-          }
-          if (in && ci == 0) finish_row(nr - 1 - item, s);
-        },
-        ring);
     if constexpr (VAR == 0) {
       if (disp) disp_reduce_cta(ds_hi, ds_lo, dq_hi, dq_lo, S.dsc, S);
     }
@@ -1833,14 +1936,15 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
 // it waits for the first only before it ends (griddepcontrol.wait, a no-op
 // in a normal launch), so that work queued after it on the stream also
 // follows the first.
-template <int VAR, bool DECODE, bool HF, bool FUSED, bool SCORE = false>
+template <int VAR, bool DECODE, bool HF, bool FUSED, bool GEN, bool SCORE = false>
 __global__ void __launch_bounds__(kThreads, SCORE    ? VD_SCORE_MIN_CTAS
+                                            : GEN    ? VD_GENERAL_MIN_CTAS
                                             : DECODE ? VD_DECODE_MIN_CTAS
                                             : HF     ? VD_HF_BLOCK_MIN_CTAS
                                                      : VD_BLOCK_MIN_CTAS)
     evict_kernel(const EvictArgs a) {
   grid_launch_dependents();
-  evict_unit<VAR, DECODE, HF, FUSED, SCORE>(a);
+  evict_unit<VAR, DECODE, HF, FUSED, SCORE, GEN>(a);
   grid_dependency_wait();
 }
 

@@ -5,17 +5,24 @@
 #include "vd_small.cuh"
 
 namespace vd {
-const void* evict_kernel_dir(bool decode, bool holefill, bool fused) {
+namespace {
+template <bool GEN>
+const void* pick(bool decode, bool holefill, bool fused) {
   const void* k[2][2][2] = {
-      {{reinterpret_cast<const void*>(&evict_kernel<1, false, false, false>),
-        reinterpret_cast<const void*>(&evict_kernel<1, false, false, true>)},
-       {reinterpret_cast<const void*>(&evict_kernel<1, false, true, false>),
-        reinterpret_cast<const void*>(&evict_kernel<1, false, true, true>)}},
-      {{reinterpret_cast<const void*>(&evict_kernel<1, true, false, false>),
-        reinterpret_cast<const void*>(&evict_kernel<1, true, false, true>)},
-       {reinterpret_cast<const void*>(&evict_kernel<1, true, true, false>),
-        reinterpret_cast<const void*>(&evict_kernel<1, true, true, true>)}}};
+      {{reinterpret_cast<const void*>(&evict_kernel<1, false, false, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<1, false, false, true, GEN>)},
+       {reinterpret_cast<const void*>(&evict_kernel<1, false, true, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<1, false, true, true, GEN>)}},
+      {{reinterpret_cast<const void*>(&evict_kernel<1, true, false, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<1, true, false, true, GEN>)},
+       {reinterpret_cast<const void*>(&evict_kernel<1, true, true, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<1, true, true, true, GEN>)}}};
   return k[decode][holefill][fused];
+}
+}  // namespace
+
+const void* evict_kernel_dir(bool decode, bool holefill, bool fused) {
+  return pick<true>(decode, holefill, fused);
 }
 
 const void* small_kernel_dir(bool decode, bool fused) {
@@ -28,6 +35,6 @@ const void* small_kernel_dir(bool decode, bool fused) {
 }
 
 const void* score_kernel_dir() {
-  return reinterpret_cast<const void*>(&evict_kernel<1, true, false, false, true>);
+  return reinterpret_cast<const void*>(&evict_kernel<1, true, false, false, true, true>);
 }
 }  // namespace vd

@@ -5,17 +5,25 @@
 #include "vd_small.cuh"
 
 namespace vd {
-const void* evict_kernel_norm(bool decode, bool holefill, bool fused) {
+namespace {
+template <bool GEN>
+const void* pick(bool decode, bool holefill, bool fused) {
   const void* k[2][2][2] = {
-      {{reinterpret_cast<const void*>(&evict_kernel<2, false, false, false>),
-        reinterpret_cast<const void*>(&evict_kernel<2, false, false, true>)},
-       {reinterpret_cast<const void*>(&evict_kernel<2, false, true, false>),
-        reinterpret_cast<const void*>(&evict_kernel<2, false, true, true>)}},
-      {{reinterpret_cast<const void*>(&evict_kernel<2, true, false, false>),
-        reinterpret_cast<const void*>(&evict_kernel<2, true, false, true>)},
-       {reinterpret_cast<const void*>(&evict_kernel<2, true, true, false>),
-        reinterpret_cast<const void*>(&evict_kernel<2, true, true, true>)}}};
+      {{reinterpret_cast<const void*>(&evict_kernel<2, false, false, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<2, false, false, true, GEN>)},
+       {reinterpret_cast<const void*>(&evict_kernel<2, false, true, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<2, false, true, true, GEN>)}},
+      {{reinterpret_cast<const void*>(&evict_kernel<2, true, false, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<2, true, false, true, GEN>)},
+       {reinterpret_cast<const void*>(&evict_kernel<2, true, true, false, GEN>),
+        reinterpret_cast<const void*>(&evict_kernel<2, true, true, true, GEN>)}}};
   return k[decode][holefill][fused];
+}
+}  // namespace
+
+// general: the score pass for any head dim (else d is 64, 128 or 256)
+const void* evict_kernel_norm(bool decode, bool holefill, bool fused, bool general) {
+  return general ? pick<true>(decode, holefill, fused) : pick<false>(decode, holefill, fused);
 }
 
 const void* small_kernel_norm(bool decode, bool fused) {
@@ -27,7 +35,8 @@ const void* small_kernel_norm(bool decode, bool fused) {
   return k[decode][fused];
 }
 
-const void* score_kernel_norm() {
-  return reinterpret_cast<const void*>(&evict_kernel<2, true, false, false, true>);
+const void* score_kernel_norm(bool general) {
+  return general ? reinterpret_cast<const void*>(&evict_kernel<2, true, false, false, true, true>)
+                 : reinterpret_cast<const void*>(&evict_kernel<2, true, false, false, false, true>);
 }
 }  // namespace vd
