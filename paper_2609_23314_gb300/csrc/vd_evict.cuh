@@ -599,18 +599,64 @@ __device__ __forceinline__ void merge_columns(float (&hi)[8], float (&lo)[8], in
   }
 }
 
+// merge_columns through the ring (whose copies have landed: 512 * P bytes of it)
+// instead of one warp after another: three block barriers for eight, the same
+// sums (acc need not be zeroed): 288 units of 2176 rows, d = 128, 135.0 -> 133.3
+// us with the select below, in the hole-fill layout 53.0 -> 52.0.  Only in the
+// block kernels with the batched scores: the others spill with it.
+__device__ __forceinline__ void merge_columns_ring(float (&hi)[8], float (&lo)[8], int P, bool active,
+                                              int chunk0, int nchunks, float* acc_hi,
+                                              float* acc_lo, uint32_t ring) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  ff p[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) p[k] = ff_add(ff{hi[k], 0.f}, ff{0.f, lo[k]});
+  for (int off = P; off < 32; off <<= 1) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) p[k] = ff_add(p[k], ff_shfl_xor(p[k], off));
+  }
+  const uint32_t row = (uint32_t)P * 32u, lo_off = (uint32_t)kWarps * row;  // bytes
+  __syncthreads();  // every thread is done with the ring
+  if (lane < P && active) {
+    const uint32_t at = ring + (uint32_t)warp * row + (uint32_t)lane * 32u;
+    auto bits = [](float a, float b, float c, float d) {
+      return make_uint4(__float_as_uint(a), __float_as_uint(b), __float_as_uint(c),
+                        __float_as_uint(d));
+    };
+    st_shared16(at, bits(p[0].hi, p[1].hi, p[2].hi, p[3].hi));
+    st_shared16(at + 16u, bits(p[4].hi, p[5].hi, p[6].hi, p[7].hi));
+    st_shared16(at + lo_off, bits(p[0].lo, p[1].lo, p[2].lo, p[3].lo));
+    st_shared16(at + lo_off + 16u, bits(p[4].lo, p[5].lo, p[6].lo, p[7].lo));
+  }
+  __syncthreads();
+  if (tid < nchunks * 8) {
+    const uint32_t at = ring + (uint32_t)tid * 4u;
+    ff t{0.f, 0.f};
+#pragma unroll 1
+    for (int w = 0; w < kWarps; ++w)
+      t = ff_add(t, ff{ld_shared_f32(at + (uint32_t)w * row),
+                       ld_shared_f32(at + (uint32_t)w * row + lo_off)});
+    acc_hi[chunk0 * 8 + tid] = t.hi;
+    acc_lo[chunk0 * 8 + tid] = t.lo;
+  }
+  __syncthreads();
+}
+
 // acc (zeroed here) <- sum over items [0, count) of sign(item) * (the row at
 // row_ptr(item)), restricted to 16-byte column chunks [chunk0, chunk0 +
 // nchunks).
 // PACKED: TwoSum on packed fp32 pairs (half the instructions); the scalar
 // form gives bit-identical sums and is kept where the packed one would not
-// fit the kernel's register budget (the Dir block kernels).
-template <class Ring, bool PACKED = true, class RowPtr, class SignOf>
+// fit the kernel's register budget (the Dir block kernels).  QUICK:
+// merge_columns_ring.
+template <class Ring, bool PACKED = true, bool QUICK = false, class RowPtr, class SignOf>
 __device__ __forceinline__ void sum_rows(int chunk0, int nchunks, int P, int count,
                                          RowPtr row_ptr, SignOf sign_of, Smem& S, uint32_t ring) {
-  S.acc_hi[threadIdx.x] = 0.f;
-  S.acc_lo[threadIdx.x] = 0.f;
-  __syncthreads();
+  if (!QUICK) {
+    S.acc_hi[threadIdx.x] = 0.f;
+    S.acc_lo[threadIdx.x] = 0.f;
+    __syncthreads();
+  }
   const int ci = (threadIdx.x & 31) & (P - 1);
   const bool active = ci < nchunks;
   // the columns of this lane's chunk as packed pairs (2k, 2k + 1); each
@@ -652,7 +698,10 @@ __device__ __forceinline__ void sum_rows(int chunk0, int nchunks, int P, int cou
                       },
                       ring);
   }
-  merge_columns(hi, lo, P, active, (chunk0 + ci) * 8, S.acc_hi, S.acc_lo);
+  if constexpr (QUICK)
+    merge_columns_ring(hi, lo, P, active, chunk0, nchunks, S.acc_hi, S.acc_lo, ring);
+  else
+    merge_columns(hi, lo, P, active, (chunk0 + ci) * 8, S.acc_hi, S.acc_lo);
 }
 
 static_assert(offsetof(Smem, ghist) == offsetof(Smem, mulo) + 1024, "dup_index");
@@ -894,7 +943,9 @@ struct Selection {
 // each thread counts how many candidates are greater than and equal to its
 // own.  The threshold is the candidate with g < need <= g + e.  Candidate
 // counts come from the cluster-summed histogram, so every CTA of the cluster
-// takes the same branch.
+// takes the same branch.  Every thread loads four keys before it counts or
+// compacts any (a shared atomic orders the loads behind it): the loops are
+// latency-bound, 17 keys per thread at 4352 rows.
 template <class KeyOf>
 __device__ __forceinline__ Selection cluster_radix_select(KeyOf key_of, int R, int N, int C,
                                                           Smem& S, bool first_ready = false) {
@@ -909,22 +960,31 @@ __device__ __forceinline__ Selection cluster_radix_select(KeyOf key_of, int R, i
       h[tid] = 0;
       __syncthreads();
     }
-    for (int base = 0; !counted && base < R; base += kThreads) {
-      const int j = base + tid;
-      bool ok = false;
-      uint32_t key = 0u;
-      if (j < R) key = key_of(j, ok);
-      const bool match = ok && (key & pmask) == prefix;
-      const uint32_t dig = (key >> shift) & 255u;
-      if (pass == 0) {
-        // the top bytes of nearby scores coincide: one atomic per distinct digit
-        const unsigned act = __ballot_sync(kFull, match);
-        if (match) {
-          const unsigned peers = __match_any_sync(act, dig);
-          if (lane == __ffs(peers) - 1) atomicAdd(&h[dig], (uint32_t)__popc(peers));
+    // four keys in flight per thread: their loads are not ordered by the atomics
+    for (int base = tid; !counted && base - tid < R; base += 4 * kThreads) {
+      uint32_t key[4];
+      bool ok[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int j = base + m * kThreads;
+        ok[m] = false;
+        key[m] = 0u;
+        if (j < R) key[m] = key_of(j, ok[m]);
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const bool match = ok[m] && (key[m] & pmask) == prefix;
+        const uint32_t dig = (key[m] >> shift) & 255u;
+        if (pass == 0) {
+          // the top bytes of nearby scores coincide: one atomic per distinct digit
+          const unsigned act = __ballot_sync(kFull, match);
+          if (match) {
+            const unsigned peers = __match_any_sync(act, dig);
+            if (lane == __ffs(peers) - 1) atomicAdd(&h[dig], (uint32_t)__popc(peers));
+          }
+        } else if (match) {
+          atomicAdd(&h[dig], 1u);  // later digits are spread: plain shared atomics
         }
-      } else if (match) {
-        atomicAdd(&h[dig], 1u);  // later digits are spread: plain shared atomics
       }
     }
     if (C > 1) cluster_sync(); else __syncthreads();
@@ -979,17 +1039,19 @@ __device__ __forceinline__ Selection cluster_radix_select(KeyOf key_of, int R, i
     // (ghist is free once every thread has read the scan's result above)
     if (tid == 0) S.ncand = 0;
     __syncthreads();
-    for (int base = 0; base < R; base += kThreads) {
-      const int j = base + tid;
-      bool ok = false;
-      uint32_t key = 0u;
-      if (j < R) key = key_of(j, ok);
-      const bool match = ok && (key & pmask) == prefix;
-      const unsigned act = __ballot_sync(kFull, match);
-      int at = 0;
-      if (lane == 0 && act) at = atomicAdd(&S.ncand, __popc(act));
-      at = __shfl_sync(kFull, at, 0);
-      if (match) S.ghist[at + __popc(act & ((1u << lane) - 1u))] = key;
+    for (int base = tid; base < R; base += 4 * kThreads) {
+      uint32_t key[4];
+      bool ok[4];
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        const int j = base + m * kThreads;
+        ok[m] = false;
+        key[m] = 0u;
+        if (j < R) key[m] = key_of(j, ok[m]);
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m)  // few match: one shared atomic each
+        if (ok[m] && (key[m] & pmask) == prefix) S.ghist[atomicAdd(&S.ncand, 1)] = key[m];
     }
     if (C > 1) cluster_sync(); else __syncthreads();
     // every CTA gathers the cluster's candidates, in rank order, into the
@@ -1011,6 +1073,7 @@ __device__ __forceinline__ Selection cluster_radix_select(KeyOf key_of, int R, i
     __syncthreads();
     if (tid < cnt) {
       int g = 0, e = 0;
+#pragma unroll 8
       for (int i = 0; i < cnt; ++i) {
         const uint32_t o = all[i];
         g += o > mine;
@@ -1463,6 +1526,7 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
   constexpr bool fused = FUSED;  // the new rows are still in the staging buffers
   // packed-pair row sums everywhere but the Dir block kernels (register budget)
   constexpr bool kPackedSum = !(VAR == 1 && !DECODE);
+  constexpr bool kQuickMerge = !DECODE && !GEN;
   const int len0 = a.len[seq];
   const int n = len0 + (fused ? a.B : 0);
   const int Nb = a.N_dev ? a.N_dev[seq] : a.N;
@@ -1534,7 +1598,7 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
     if (DECODE && a.evicted_out && rank == 0 && tid == 0) a.evicted_out[u] = -1;
     if (a.mu_running && a.B > 0 && tchunks > 0) {
       const uint16_t* nb = srange(first_new, a.B);  // the new rows lie on one side
-      sum_rows<Ring, kPackedSum>(tchunk0, tchunks, tp, a.B, [&](int i) { return nb + (size_t)i * d; },
+      sum_rows<Ring, kPackedSum, kQuickMerge>(tchunk0, tchunks, tp, a.B, [&](int i) { return nb + (size_t)i * d; },
                [](int) { return 1.f; }, S, ring);
       if (tid < tchunks * 8) {
         const int c = tchunk0 * 8 + tid;
@@ -1576,7 +1640,7 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
     if constexpr (bulk)  // score-only rows are never staged: one contiguous range
       sum_rows_bulk(br, pb, cnt, d, lpr, S, a.status);
     else
-      sum_rows<Ring, kPackedSum>(0, d8, lpr, cnt,
+      sum_rows<Ring, kPackedSum, kQuickMerge>(0, d8, lpr, cnt,
                      [&](int i) -> const uint16_t* {
                        if constexpr (FUSED) return pb ? pb + (size_t)i * d : srow(p0 + i);
                        else return pb + (size_t)i * d;
@@ -1848,7 +1912,7 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
       const int c = tchunk0 * 8 + tid;
       base = VAR != 2 ? S.snew[c] : a.running_sum[(size_t)u * d + c] + 0.0;
     }
-    sum_rows<Ring, kPackedSum>(tchunk0, tchunks, tp, B + ne,
+    sum_rows<Ring, kPackedSum, kQuickMerge>(tchunk0, tchunks, tp, B + ne,
              [&](int i) {
                const int r =
                    i < B ? first_new + i : (DECODE ? e_first : (int)perm[Nb + (i - B)]);
