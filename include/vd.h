@@ -46,9 +46,9 @@
  *   one wave at one CTA per unit but has more units than the GPU has SMs
  *   runs the eviction kernel as two launches over disjoint units, the second
  *   a programmatic dependent of the first, so that no SM carries a whole
- *   unit more than the others.  A short cache (capacity <= 1024,
+ *   unit more than the others.  A short cache (capacity <= 256,
  *   4 * capacity * head_dim <= 64 KB, at most 16 units per sequence, at most
- *   two units per SM) takes a kernel that keeps the unit in shared memory
+ *   one unit per SM) takes a kernel that keeps the unit in shared memory
  *   and updates the lengths itself: one launch in all.  Results follow the
  *   same rules either way, and every call can be captured in a CUDA graph.
  */

@@ -500,12 +500,13 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
 
 // The short-cache kernel (vd_small.cuh) takes a block or decode event when
 // the unit's K and V rows fit in shared memory with room to spare
-// (capacity * head_dim * 4 bytes <= kSmallRowBytes, capacity <= 1024), a
-// sequence's units fit in one cluster (<= 16), the launch is at most two
-// waves of one CTA per SM, and no scoring option, hole-fill layout or forced
-// cluster size (VD_CLUSTER_SIZE) is asked for.  VD_SMALL_PATH=0 turns it
-// off.  The choice depends on the shape only, so the fused and two-call
-// forms, block and decode, take the same kernel.
+// (capacity * head_dim * 4 bytes <= kSmallRowBytes, capacity <=
+// vd::kSmallMaxRows), a sequence's units fit in one cluster (<= 16), the launch
+// is at most one CTA per SM (60 units of 160 rows 9.5 us against 11.9 with the
+// resident kernel, 200 units 13.2 against 12.9), and no scoring option, hole-fill
+// layout or forced cluster size (VD_CLUSTER_SIZE) is asked for.
+// VD_SMALL_PATH=0 turns it off.  The choice depends on the shape only, so the
+// fused and two-call forms, block and decode, take the same kernel.
 constexpr size_t kSmallRowBytes = 64 * 1024;
 
 bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* weights,
@@ -515,7 +516,7 @@ bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* w
   if ((off && std::atoi(off) == 0) || std::getenv("VD_CLUSTER_SIZE")) return false;
   const int ups = c->n_layer * c->n_kv_head;
   const long long units = (long long)c->n_seq * ups;
-  if (ups > 16 || c->capacity > vd::kSmallMaxRows || units > 2LL * st.sms) return false;
+  if (ups > 16 || c->capacity > vd::kSmallMaxRows || units > st.sms) return false;
   if ((size_t)c->capacity * c->head_dim * 4 > kSmallRowBytes) return false;
   return vd::small_layout(c->capacity, c->head_dim).total <= (size_t)st.smem_optin;
 }

@@ -273,9 +273,10 @@ __device__ __forceinline__ void resident_score_fast(uint32_t buf, int ca, int cb
 // a time, per row the arithmetic of the streaming kernel's general path (lanes
 // added at distance 1, 2, 4, ...).  With at least as many lanes as rows the
 // last reduction hands each of the first lanes one row.
-template <int VAR, class Finish>
+// Sm: ResSmem or SmallSmem (the mean in column order, and Dir's factors).
+template <int VAR, class Sm, class Finish>
 __device__ __forceinline__ void resident_score_general(uint32_t buf, int ca, int cb, int d, int lpr,
-                                                       const ResSmem& S, Finish finish) {
+                                                       const Sm& S, Finish finish) {
   constexpr int kBatch = VAR == 1 ? 2 : 4, kLog = VAR == 1 ? 1 : 2;
   const int ci = (threadIdx.x & 31) & (lpr - 1), g = threadIdx.x / lpr, ng = kThreads / lpr;
   const bool active = ci < (d >> 3);

@@ -14,11 +14,18 @@
 //              w = v - (|v|/|m|) m, Norm |v|^2, as in the fused kernel
 //   3. select  rank_j = #{i : key_i > key_j} + #{i < j : key_i == key_j};
 //              row j survives iff rank_j < N (Eq. eviction, ties to the
-//              lower slot), O(n^2 / 256) comparisons per thread
+//              lower slot), n comparisons per thread, four keys per load
 //   4. list    kept slots ascending (a block prefix sum), then the evicted
 //   5. sum     running mode: S + sum(appended rows) - sum(evicted rows)
 //   6. move    rows [first moved, N) written from the shared-memory copy,
 //              so the in-place gather has no read-after-write hazard
+//
+// Bound by the latency of these steps.  The rows arrive by bulk copies (K while
+// V is scored), the running sum is read before they land, rows are scored four
+// at a time and compacted two at a time: 2 units of 160 rows, d = 64, 9.2 ->
+// 8.1 us a call.  Up to 256 rows: beyond, the comparisons cost more than the
+// resident kernel's histogram and second launch (d = 64, 256 rows 9.9 us against
+// 11.8; d = 32, 384 rows 14.4 against 12.0; d = 16, 1000 rows 45.7 against 13.0).
 //
 // Same validation, outputs and status codes as the fused kernel; no
 // hole-fill layout, attention weights, sigma or key-side rule (those calls
@@ -27,22 +34,22 @@
 
 #include <cstdint>
 
-#include "vd_evict.cuh"
+#include "vd_resident.cuh"
 
 namespace vd {
 
-constexpr int kSmallMaxRows = 1024;
+constexpr int kSmallMaxRows = kThreads;  // one row per thread in the rank select
 
 struct SmallSmem {
   float mu[256];
   float mulo[256];     // mean = mu + mulo (natural column order)
   float part_hi[256];  // column-sum partials, [part][column]
   float part_lo[256];
+  unsigned long long bar[2];  // V rows, K rows
   int scan[kWarps];
   float fsh[kWarps];
   float inv_mnorm;
   int mu_zero;
-  int e_first;
 };
 
 struct SmallLayout {
@@ -72,6 +79,7 @@ __device__ __forceinline__ ff small_column_sum(int d, int count, RowOf row_of, S
   const int col = tid % d, part = tid / d;
   float hi = 0.f, lo = 0.f;
   if (part < P)
+#pragma unroll 4
     for (int i = part; i < count; i += P)
       ff_accumulate(hi, lo, sign_of(i) * __uint_as_float((uint32_t)row_of(i)[col] << 16));
   if (part < P) {
@@ -99,12 +107,19 @@ struct SmallArgs {
 template <int VAR, bool DECODE, bool FUSED>
 __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArgs sa) {
   const EvictArgs& a = sa.e;
-  // launched as a programmatic dependent: wait for the previous kernel on the
-  // stream before reading anything, and let the next one be scheduled
-  grid_dependency_wait();
-  grid_launch_dependents();
+  // launched as a programmatic dependent: set up the barriers, wait for the
+  // previous kernel on the stream before reading anything, and let the next one
+  // be scheduled
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SmallSmem& S = *reinterpret_cast<SmallSmem*>(smem_raw);
+  const uint32_t bar_v = smem_addr(&S.bar[0]), bar_k = smem_addr(&S.bar[1]);
+  if (threadIdx.x == 0) {
+    mbar_init(bar_v, 1);
+    mbar_init(bar_k, 1);
+    fence_mbar_init();
+  }
+  grid_dependency_wait();
+  grid_launch_dependents();
   const int d = a.d, d8 = d >> 3, cap = a.capacity;
   const SmallLayout L = small_layout(cap, d);
   uint16_t* Vs = reinterpret_cast<uint16_t*>(smem_raw + L.v);
@@ -144,24 +159,30 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
   const int first_new = n - a.B;
 
   if (ok) {
-    // ---- the unit's rows into shared memory (cache rows below len0, the
-    // staging rows above it when fused) ---------------------------------
+    // ---- the unit's rows into shared memory: one bulk copy per tensor of the
+    // cache rows, one of the staged ones; K, which only the compaction reads,
+    // lands while V is scored ---------------------------------------------
     const uint32_t vs_a = smem_addr(Vs), ks_a = smem_addr(Ks);
-    for (int c = tid; c < n * d8; c += kThreads) {
-      const int r = c / d8, col = (c - r * d8) * 8;
-      const bool staged = FUSED && r >= len0;
-      const size_t go = (size_t)(staged ? r - len0 : r) * d + col;
-      cp_async16(vs_a + (uint32_t)(r * d + col) * 2u, (staged ? vnu : vb) + go);
-      cp_async16(ks_a + (uint32_t)(r * d + col) * 2u, (staged ? knu : kb) + go);
-    }
-    cp_async_commit();
-    cp_async_wait<0>();
-    __syncthreads();
-    auto vrow = [&](int r) { return Vs + (size_t)r * d; };
     double* rsu = a.mu_running ? a.running_sum + (size_t)u * d : nullptr;
+    if (tid == 0) {
+      const uint32_t row = (uint32_t)d * 2u, old = (uint32_t)len0 * row, all = (uint32_t)n * row;
+      for (int t = 0; t < 2; ++t) {
+        const uint32_t bar = t ? bar_k : bar_v, dst = t ? ks_a : vs_a;
+        mbar_expect_tx(bar, all);
+        if (old > 0) bulk_g2s(dst, t ? kb : vb, old, bar);
+        if (FUSED) bulk_g2s(dst + old, t ? knu : vnu, all - old, bar);
+      }
+    }
+    // the running sum and 1 / n do not wait for the rows
+    const double rs_old = rsu && tid < d ? rsu[tid] : 0.0;
+    const double dn = (double)n, rn = tid < d ? 1.0 / dn : 0.0;
+    __syncthreads();
+    mbar_wait(bar_v, 0u, a.status);
+    auto vrow = [&](int r) { return Vs + (size_t)r * d; };
 
     if (!evict) {
       // ---- nothing to evict: append (fused), running sum += appended rows --
+      mbar_wait(bar_k, 0u, a.status);
       if (FUSED)
         for (int c = tid; c < a.B * d8; c += kThreads) {
           const int r = len0 + c / d8, col = (c % d8) * 8;
@@ -174,7 +195,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
       if (rsu && a.B > 0) {
         const ff t = small_column_sum(d, a.B, [&](int i) { return vrow(first_new + i); },
                                       [](int) { return 1.f; }, S);
-        if (tid < d) rsu[tid] = rsu[tid] + (double)t.hi + (double)t.lo;
+        if (tid < d) rsu[tid] = rs_old + (double)t.hi + (double)t.lo;
       }
     } else {
       // ---- 1. mean ----------------------------------------------------
@@ -187,9 +208,10 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
                                       [](int) { return 1.f; }, S);
         if (tid < d) {
           double sum = (double)t.hi + (double)t.lo;
-          if (run) sum += rsu[tid];
+          if (run) sum += rs_old;
           s_app = sum;
-          const double m = sum / (double)n;
+          // sum / n as a product with the reciprocal and one correction
+          const double m0 = sum * rn, m = fma(fma(-m0, dn, sum), rn, m0);
           const float mh = (float)m;
           S.mu[tid] = mh;
           S.mulo[tid] = (float)(m - (double)mh);
@@ -206,94 +228,45 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
         }
       }
       // ---- 2. scores: lpr lanes per row, one 16-byte chunk each ----------
-      const int lpr = a.lpr, ci = lane & (lpr - 1), g = tid / lpr, ng = kThreads / lpr;
-      const bool active = ci < d8;
-      float m8[8], l8[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        m8[k] = (VAR != 2 && active) ? S.mu[ci * 8 + k] : 0.f;
-        l8[k] = (VAR != 2 && active) ? S.mulo[ci * 8 + k] : 0.f;
-      }
-      const bool mu_zero = VAR == 1 && S.mu_zero;
-      const float inv_mnorm = VAR == 1 ? S.inv_mnorm : 0.f;
       float* sc_out = a.scores_out ? a.scores_out + (size_t)u * cap : nullptr;
-      for (int base = 0; base < n; base += ng) {
-        const int j = base + g;
-        const bool in = j < n;
-        uint4 q = make_uint4(0u, 0u, 0u, 0u);
-        if (in && active) q = ld_shared16(vs_a + (uint32_t)(j * d + ci * 8) * 2u);
-        float x[8];
-        unpack8(q, x);
-        float sc;
-        if (VAR == 0) {
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const float dv = (x[k] - m8[k]) - l8[k];
-            acc = fmaf(dv, dv, acc);
-          }
-          for (int off = 1; off < lpr; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
-          sc = sqrtf(acc);
-        } else if (VAR == 2) {
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) acc = fmaf(x[k], x[k], acc);
-          for (int off = 1; off < lpr; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
-          sc = sqrtf(acc);
-        } else {
-          float nv = 0.f;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) nv = fmaf(x[k], x[k], nv);
-          for (int off = 1; off < lpr; off <<= 1) nv += __shfl_xor_sync(kFull, nv, off);
-          const float lam = sqrtf(nv) * inv_mnorm;
-          float acc = 0.f;
-#pragma unroll
-          for (int k = 0; k < 8; ++k) {
-            const float w = fmaf(-lam, l8[k], fmaf(-lam, m8[k], x[k]));
-            acc = fmaf(w, w, acc);
-          }
-          for (int off = 1; off < lpr; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
-          sc = (nv > 0.f && !mu_zero) ? (0.5f * acc) / nv : 1.f;
-        }
-        if (in && ci == 0) {
-          bool bad;
-          keys[j] = score_key(sc, bad);
-          if (bad) record_status(a.status, kStNonfinite);
-          if (sc_out) sc_out[j] = sc;
-        }
-      }
+      resident_score_general<VAR>(vs_a, 0, n, d, a.lpr, S, [&](int j, float sc) {
+        bool bad;
+        keys[j] = score_key(sc, bad);
+        if (bad) record_status(a.status, kStNonfinite);
+        if (sc_out) sc_out[j] = sc;
+      });
       __syncthreads();
 
       // ---- 3./4. rank select and the kept list -------------------------
-      // thread t owns rows [t * ch, t * ch + ch), so prefix sums follow slot
-      // order (ties go to the lower slot)
-      const int ch = (n + kThreads - 1) / kThreads;
-      const int c0 = min(n, tid * ch), c1 = min(n, c0 + ch);
-      unsigned keep_bits = 0u;  // ch <= kSmallMaxRows / kThreads = 4
-      int nkeep = 0;
-      for (int j = c0; j < c1; ++j) {
-        const uint32_t kj = keys[j];
+      // thread t owns row t, so prefix sums follow slot order (ties go to the
+      // lower slot)
+      bool keep = false;
+      if (tid < n) {
+        const uint32_t kj = keys[tid];
         int rank_j = 0;
-        for (int i = 0; i < n; ++i) {
-          const uint32_t ki = keys[i];
-          rank_j += (ki > kj) | ((ki == kj) & (i < j));
+        auto rank_against = [&](uint32_t ki, int i) {
+          rank_j += (ki > kj) | ((ki == kj) & (i < tid));
+        };
+        const uint4* k4 = reinterpret_cast<const uint4*>(keys);  // four keys per load
+#pragma unroll 4
+        for (int i = 0; i < (n >> 2); ++i) {
+          const uint4 k = k4[i];
+          rank_against(k.x, 4 * i);
+          rank_against(k.y, 4 * i + 1);
+          rank_against(k.z, 4 * i + 2);
+          rank_against(k.w, 4 * i + 3);
         }
-        if (rank_j < Nb) {
-          keep_bits |= 1u << (j - c0);
-          ++nkeep;
-        }
+        for (int i = n & ~3; i < n; ++i) rank_against(keys[i], i);
+        keep = rank_j < Nb;
       }
       int total_kept;
-      int kp = block_exclusive_scan(nkeep, S.scan, total_kept);
-      for (int j = c0; j < c1; ++j) {
-        const bool keep = (keep_bits >> (j - c0)) & 1u;
-        const int pos = keep ? kp : Nb + (j - kp);
-        kp += keep;
-        if ((unsigned)pos >= (unsigned)n || total_kept != Nb) {  // self-check
+      const int kept_at = block_exclusive_scan(keep ? 1 : 0, S.scan, total_kept);
+      if (tid < n) {
+        const int pos = keep ? kept_at : Nb + (tid - kept_at);
+        if ((unsigned)pos >= (unsigned)n || total_kept != Nb)  // self-check
           record_status(a.status, kStInternal);
-          continue;
-        }
-        perm[pos] = (uint16_t)j;
+        else
+          perm[pos] = (uint16_t)tid;
       }
       __syncthreads();
       // perm entries index the shared-memory copy: clamped to [0, n) so that
@@ -317,12 +290,27 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
       // ---- 6. compaction from the shared-memory copy ---------------------
       // (fused: the kept new rows below the budget are written too)
       const int r_begin = FUSED ? min(e_first, len0) : e_first;
-      for (int c = tid; c < (Nb - r_begin) * d8; c += kThreads) {
-        const int r = r_begin + c / d8, col = (c % d8) * 8;
-        const int src = slot(r);
-        st16(kb + (size_t)r * d + col, ld_shared16(ks_a + (uint32_t)(src * d + col) * 2u));
-        st16(vb + (size_t)r * d + col, ld_shared16(vs_a + (uint32_t)(src * d + col) * 2u));
-      }
+      mbar_wait(bar_k, 0u, a.status);
+      const int ci = lane & (a.lpr - 1), g = tid / a.lpr, ng = kThreads / a.lpr;
+      const unsigned char* vp = reinterpret_cast<const unsigned char*>(Vs) + ci * 16;
+      const unsigned char* kp = reinterpret_cast<const unsigned char*>(Ks) + ci * 16;
+      if (ci < d8)
+        for (int r0 = r_begin + g; r0 < Nb; r0 += 2 * ng) {
+          uint4 qk[2], qv[2];  // two rows of each tensor in flight
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            const size_t src = (size_t)slot(min(r0 + m * ng, Nb - 1)) * d * 2;
+            qk[m] = *reinterpret_cast<const uint4*>(kp + src);
+            qv[m] = *reinterpret_cast<const uint4*>(vp + src);
+          }
+#pragma unroll
+          for (int m = 0; m < 2; ++m) {
+            if (r0 + m * ng >= Nb) break;
+            const size_t dst = (size_t)(r0 + m * ng) * d + ci * 8;
+            st16(kb + dst, qk[m]);
+            st16(vb + dst, qv[m]);
+          }
+        }
     }
   }
 
