@@ -39,17 +39,17 @@
  *   to about 1e-12 of the data's scale.  Every score's rounding error is
  *   relative to the score itself (a few 1e-7 in practice).  Ranking: a NaN
  *   score ranks below every number, +0 and -0 are equal.
- * - Launches: one eviction kernel per call (calls of few units take one that
- *   keeps a unit's scored rows in shared memory), plus a one-thread-per-sequence
- *   length update (a programmatic dependent launch of the eviction, all on
- *   `stream`).  A hole-fill block eviction or a score-only call that fits
- *   one wave at one CTA per unit but has more units than the GPU has SMs
- *   runs the eviction kernel as two launches over disjoint units, the second
- *   a programmatic dependent of the first, so that no SM carries a whole
+ * - Launches: one eviction kernel per call (calls of few or small units take
+ *   one that keeps a unit's scored rows in shared memory), plus a
+ *   one-thread-per-sequence length update (a programmatic dependent launch of
+ *   the eviction, all on `stream`).  A hole-fill block eviction or a score-only
+ *   call that fits one wave at one CTA per unit but has more units than the GPU
+ *   has SMs runs the eviction kernel as two launches over disjoint units, the
+ *   second a programmatic dependent of the first, so that no SM carries a whole
  *   unit more than the others.  A short cache (capacity <= 256,
- *   4 * capacity * head_dim <= 64 KB, at most 16 units per sequence, at most
- *   one unit per SM) takes a kernel that keeps the unit in shared memory
- *   and updates the lengths itself: one launch in all.  Results follow the
+ *   4 * capacity * head_dim <= 64 KB) takes a kernel that keeps the unit's K
+ *   and V in shared memory and, with at most 16 units per sequence and one unit
+ *   per SM, updates the lengths itself: one launch in all.  Results follow the
  *   same rules either way, and every call can be captured in a CUDA graph.
  */
 #ifndef VD_H

@@ -501,10 +501,10 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
 // The short-cache kernel (vd_small.cuh) takes a block or decode event when
 // the unit's K and V rows fit in shared memory with room to spare
 // (capacity * head_dim * 4 bytes <= kSmallRowBytes, capacity <=
-// vd::kSmallMaxRows), a sequence's units fit in one cluster (<= 16), the launch
-// is at most one CTA per SM (60 units of 160 rows 9.5 us against 11.9 with the
-// resident kernel, 200 units 13.2 against 12.9), and no scoring option, hole-fill
-// layout or forced cluster size (VD_CLUSTER_SIZE) is asked for.
+// vd::kSmallMaxRows) and no scoring option, hole-fill layout or forced cluster
+// size (VD_CLUSTER_SIZE) is asked for.  It sets the lengths itself where a
+// sequence's units fit in one cluster (<= 16) and the launch is at most one CTA
+// per SM (60 units of 160 rows 9.5 us; 200 units 13.2, and 12.9 without).
 // VD_SMALL_PATH=0 turns it off.  The choice depends on the shape only, so the
 // fused and two-call forms, block and decode, take the same kernel.
 constexpr size_t kSmallRowBytes = 64 * 1024;
@@ -514,9 +514,7 @@ bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* w
   if (score_only || holefill || weights || disp_out || score_k) return false;
   const char* off = std::getenv("VD_SMALL_PATH");
   if ((off && std::atoi(off) == 0) || std::getenv("VD_CLUSTER_SIZE")) return false;
-  const int ups = c->n_layer * c->n_kv_head;
-  const long long units = (long long)c->n_seq * ups;
-  if (ups > 16 || c->capacity > vd::kSmallMaxRows || units > st.sms) return false;
+  if (c->capacity > vd::kSmallMaxRows) return false;
   if ((size_t)c->capacity * c->head_dim * 4 > kSmallRowBytes) return false;
   return vd::small_layout(c->capacity, c->head_dim).total <= (size_t)st.smem_optin;
 }
@@ -577,13 +575,18 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
 // wins where the streaming kernel has too few rows per SM to hide its own, and
 // loses once several waves of clusters follow one another (288 units of 2176
 // rows, d = 128: 167 us against 136).  C is the largest size, up to 12, that
-// leaves a CTA at least 64 rows and the launch at most two CTAs per SM, and
-// whose clusters form one wave.  Measured, streaming / resident, d = 128,
+// leaves a CTA at least 64 rows and the launch at most two CTAs per SM (decode,
+// which has fewer phases: three), and whose clusters form one wave.  Measured, streaming / resident, d = 128,
 // n = 2176: 8 units 29.0 / 19.6 us (C = 12; C = 8 20.9), 16 units 31.5 / 22.1
 // (C = 10), 32 units 35.1 / 29.3 (C = 8; C = 4 30.6); n = 1152: 96 units
 // 57.2 / 33.3 (C = 3; C = 4, 2.5 CTAs per SM, 50.3).  Both tensors get a
 // buffer where that keeps the wave (8 units 17.6 us in the kernel against
-// 20.3).  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
+// 20.3).  More units, or larger ones: C = 1 where three CTAs share an SM (decode:
+// two), in any number of waves, since a small unit is only its phases in either
+// kernel.  us, streaming / resident: d = 64, 340 rows, 320 units 26.8 / 22.4, 4800
+// units 208 / 182; d = 96, 240 rows, 1600 units 105 / 86 (340 rows, two CTAs per
+// SM, 110 / 127); decode, d = 128, 301 rows, 640 units 42.9 / 33.7, 4800 units
+// 197 / 172 (451 rows, one CTA per SM, 249 / 328).  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
 // c CTAs (100 + c: with both buffers), for tests.  Returns C, or 0.
 constexpr int kResidentKind = 4;  // and 5: with the running mean
 constexpr int kResidentMinRows = 64;
@@ -593,7 +596,6 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
   const char* env = std::getenv("VD_RESIDENT");
   const int want = env ? std::atoi(env) : -1;
   if (want == 0 || std::getenv("VD_CLUSTER_SIZE") || capacity > 32768) return 0;
-  if (want < 0 && units > 2LL * st.sms) return 0;
   const int kind = kResidentKind + (running ? 1 : 0);
   {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -622,10 +624,14 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
     both = want >= 100;
     if (c < 1 || c > vd::kResMaxCluster || at_once(c, both) < 1) c = 0;
   } else {
-    const long long most = std::min<long long>(2LL * st.sms / units, capacity / kResidentMinRows);
-    for (c = (int)std::max(1LL, std::min(12LL, most)); c >= 1; --c)
-      if (at_once(c, false) >= units) break;
-    both = c >= 1 && at_once(c, true) >= units;
+    const long long room = (decode ? 3LL : 2LL) * st.sms;
+    if (units <= room) {
+      const long long most = std::min<long long>(room / units, capacity / kResidentMinRows);
+      for (c = (int)std::max(1LL, std::min(12LL, most)); c >= 1; --c)
+        if (at_once(c, false) >= units) break;
+      both = c >= 1 && at_once(c, true) >= units;
+    }
+    if (c < 1 && at_once(1, false) >= (decode ? 2LL : 3LL) * st.sms) c = 1;
   }
   const size_t smem = c >= 1 ? smem_of(c, both) : 0;
   std::lock_guard<std::mutex> lk(g_mu);
@@ -728,15 +734,19 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     return VD_OK;
   };
   if (use_small(c, score_only, holefill, weights, disp_out, score_k, *st)) {
-    // one launch: the kernel also sets the sequences' lengths
-    // grid: n_seq clusters of units_per_seq CTAs, one CTA per unit
     const void* sk = small_kernel(var, decode, fused);
     const size_t ssmem = vd::small_layout(c->capacity, c->head_dim).total;
+    // few units: n_seq clusters of units_per_seq CTAs (one CTA per unit), which
+    // also set the sequences' lengths: one launch
     a.cluster = a.units_per_seq;
-    if (cached_fits(sk, c->n_seq, a.cluster, ssmem, *st)) {
-      const vd::SmallArgs sa{a, (int32_t)units};
+    if (a.cluster <= 16 && units <= st->sms && cached_fits(sk, c->n_seq, a.cluster, ssmem, *st)) {
+      const vd::SmallArgs sa{a, (int32_t)units, 1};
       return launch(sk, c->n_seq, a.cluster, ssmem, &sa, s, true);
     }
+    a.cluster = 1;
+    const vd::SmallArgs sa{a, (int32_t)units, 0};
+    r = launch(sk, units, 1, ssmem, &sa, s, true);
+    return r != VD_OK ? r : clamp_lengths();
   }
   size_t smem = 0;
   long long solo = 0;

@@ -2,19 +2,21 @@
 // fused kernel's machinery (multi-pass radix select, streaming rings, the
 // separate length update) costs more than the work itself.
 //
-// One CTA per (sequence, layer, KV head) unit; the CTAs of one sequence form
-// one thread-block cluster (units_per_seq <= 16), so that after a cluster
-// barrier the sequence's length can be written by the kernel itself: one
-// launch per event.  The unit's n rows of K and V are copied into shared
+// One CTA per (sequence, layer, KV head) unit.  In a launch of few units the
+// CTAs of one sequence form one thread-block cluster (units_per_seq <= 16), so
+// that after a cluster barrier the sequence's length can be written by the
+// kernel itself: one launch per event.  With more units the length update is a
+// launch of its own.  The unit's n rows of K and V are copied into shared
 // memory once; everything after that reads shared memory:
 //
 //   1. mean    double-float column sums (running mode: the caller's fp64 sum
 //              S plus the appended rows), kept as an fp32 part and remainder
 //   2. score   L2 ((v - hi) - lo)^2, Dir |w|^2 / (2 |v|^2) with
 //              w = v - (|v|/|m|) m, Norm |v|^2, as in the fused kernel
-//   3. select  rank_j = #{i : key_i > key_j} + #{i < j : key_i == key_j};
-//              row j survives iff rank_j < N (Eq. eviction, ties to the
-//              lower slot), n comparisons per thread, four keys per load
+//   3. select  decode: an arg-min over (key, -slot); block:
+//              rank_j = #{i : key_i > key_j} + #{i < j : key_i == key_j}, row
+//              j survives iff rank_j < N (Eq. eviction, ties to the lower
+//              slot), n comparisons per thread, four keys per load
 //   4. list    kept slots ascending (a block prefix sum), then the evicted
 //   5. sum     running mode: S + sum(appended rows) - sum(evicted rows)
 //   6. move    rows [first moved, N) written from the shared-memory copy,
@@ -26,6 +28,9 @@
 // 8.1 us a call.  Up to 256 rows: beyond, the comparisons cost more than the
 // resident kernel's histogram and second launch (d = 64, 256 rows 9.9 us against
 // 11.8; d = 32, 384 rows 14.4 against 12.0; d = 16, 1000 rows 45.7 against 13.0).
+// With many units three CTAs share an SM; us, streaming kernel / this one: d =
+// 128, 128 rows, 320 units 23.7 / 15.7, 1600 units 64 / 42, 4800 units 179 / 108;
+// decode, 101 rows, 1600 units 50 / 29.
 //
 // Same validation, outputs and status codes as the fused kernel; no
 // hole-fill layout, attention weights, sigma or key-side rule (those calls
@@ -46,6 +51,7 @@ struct SmallSmem {
   float part_hi[256];  // column-sum partials, [part][column]
   float part_lo[256];
   unsigned long long bar[2];  // V rows, K rows
+  unsigned long long best[kWarps];
   int scan[kWarps];
   float fsh[kWarps];
   float inv_mnorm;
@@ -98,6 +104,7 @@ __device__ __forceinline__ ff small_column_sum(int d, int count, RowOf row_of, S
 struct SmallArgs {
   EvictArgs e;
   int32_t n_units;  // n_seq * units_per_seq: the grid's CTAs
+  int32_t set_len;  // 1: clusters of a sequence's units, which set its length here
 };
 
 // VAR: 0 L2, 1 Dir, 2 Norm.  DECODE: the decode entry points (n <= N + 1);
@@ -238,41 +245,58 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
       __syncthreads();
 
       // ---- 3./4. rank select and the kept list -------------------------
-      // thread t owns row t, so prefix sums follow slot order (ties go to the
-      // lower slot)
-      bool keep = false;
-      if (tid < n) {
-        const uint32_t kj = keys[tid];
-        int rank_j = 0;
-        auto rank_against = [&](uint32_t ki, int i) {
-          rank_j += (ki > kj) | ((ki == kj) & (i < tid));
-        };
-        const uint4* k4 = reinterpret_cast<const uint4*>(keys);  // four keys per load
-#pragma unroll 4
-        for (int i = 0; i < (n >> 2); ++i) {
-          const uint4 k = k4[i];
-          rank_against(k.x, 4 * i);
-          rank_against(k.y, 4 * i + 1);
-          rank_against(k.z, 4 * i + 2);
-          rank_against(k.w, 4 * i + 3);
-        }
-        for (int i = n & ~3; i < n; ++i) rank_against(keys[i], i);
-        keep = rank_j < Nb;
-      }
-      int total_kept;
-      const int kept_at = block_exclusive_scan(keep ? 1 : 0, S.scan, total_kept);
-      if (tid < n) {
-        const int pos = keep ? kept_at : Nb + (tid - kept_at);
-        if ((unsigned)pos >= (unsigned)n || total_kept != Nb)  // self-check
-          record_status(a.status, kStInternal);
-        else
-          perm[pos] = (uint16_t)tid;
-      }
-      __syncthreads();
       // perm entries index the shared-memory copy: clamped to [0, n) so that
       // even after a failed self-check no access leaves it
-      auto slot = [&](int i) { return min((int)perm[i], n - 1); };
-      const int e_first = slot(Nb);  // the lowest evicted slot
+      int e_first;  // the lowest evicted slot
+      if (DECODE) {
+        // one row goes: the lowest key, the highest slot among equal ones
+        unsigned long long best = ~0ull;
+        if (tid < n)
+          best = ((unsigned long long)keys[tid] << 32) | (unsigned long long)(0xffffffffu - (unsigned)tid);
+        best = warp_min_u64(best);
+        if (lane == 0) S.best[tid >> 5] = best;
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) best = S.best[w] < best ? S.best[w] : best;
+        e_first = min((int)(0xffffffffu - (unsigned)(best & 0xffffffffull)), n - 1);
+      } else {
+        // thread t owns row t, so prefix sums follow slot order (ties go to the
+        // lower slot)
+        bool keep = false;
+        if (tid < n) {
+          const uint32_t kj = keys[tid];
+          int rank_j = 0;
+          auto rank_against = [&](uint32_t ki, int i) {
+            rank_j += (ki > kj) | ((ki == kj) & (i < tid));
+          };
+          const uint4* k4 = reinterpret_cast<const uint4*>(keys);  // four keys per load
+#pragma unroll 4
+          for (int i = 0; i < (n >> 2); ++i) {
+            const uint4 k = k4[i];
+            rank_against(k.x, 4 * i);
+            rank_against(k.y, 4 * i + 1);
+            rank_against(k.z, 4 * i + 2);
+            rank_against(k.w, 4 * i + 3);
+          }
+          for (int i = n & ~3; i < n; ++i) rank_against(keys[i], i);
+          keep = rank_j < Nb;
+        }
+        int total_kept;
+        const int kept_at = block_exclusive_scan(keep ? 1 : 0, S.scan, total_kept);
+        if (tid < n) {
+          const int pos = keep ? kept_at : Nb + (tid - kept_at);
+          if ((unsigned)pos >= (unsigned)n || total_kept != Nb)  // self-check
+            record_status(a.status, kStInternal);
+          else
+            perm[pos] = (uint16_t)tid;
+        }
+        __syncthreads();
+        e_first = min((int)perm[Nb], n - 1);
+      }
+      auto slot = [&](int i) {
+        if (DECODE) return min(i < Nb ? i + (i >= e_first) : e_first, n - 1);
+        return min((int)perm[i], n - 1);
+      };
 
       // ---- outputs --------------------------------------------------------
       if (a.kept_out)
@@ -315,6 +339,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
   }
 
   // ---- the sequence's new length, once every unit of it has read len -----
+  if (!sa.set_len) return;  // a launch of its own does it
   if (C > 1) cluster_sync(); else __syncthreads();
   if (ok && (evict || FUSED) && rank == 0 && tid == 0 && u + C <= sa.n_units)
     a.len[seq] = evict ? Nb : n;

@@ -246,3 +246,41 @@ def test_nan_row_is_reported_and_evicted_first(orc):
     assert np.isnan(s0[37]) and np.array_equal(kh[0], orc.select_top_n(s0, N))
     s1 = orc.scores(pre_v[1, :n], oracle.NORM)
     assert np.array_equal(kh[1], orc.select_top_n(s1, N))
+
+
+# ---------------------------------------------------------------------------
+# more units than one launch's clusters or SMs hold: the same kernel without
+# the cluster, the lengths set by a launch of its own
+# ---------------------------------------------------------------------------
+@pytest.mark.parametrize("decode", [False, True], ids=["block", "decode"])
+@pytest.mark.parametrize("shape", [(3, 5, 4, 64, 256), (17, 2, 5, 24, 90), (2, 1, 17, 8, 31)],
+                         ids=["60", "170", "34"])
+def test_many_units_match_the_streaming_kernel(decode, shape, monkeypatch):
+    n_seq, L, H, d, cap = shape
+    B = 1 if decode else 7
+    N = cap - B
+    lens = [N - (s % 3 == 2) * B for s in range(n_seq)]   # some sequences do not evict
+    base = filled_cache(n_seq, L, H, cap, d, lens, seed=cap, dup_fraction=0.2)
+    k, v = wl.TokenStream("gauss_outlier", base.units, d, seed=5).next(B)
+    us = base.unit_shape()
+    k, v = k.view(us + (B, d)).contiguous(), v.view(us + (B, d)).contiguous()
+    got = []
+    for small in ("1", "0"):
+        monkeypatch.setenv("VD_SMALL_PATH", small)
+        monkeypatch.setenv("VD_RESIDENT", "0")
+        c = vd.Cache(base.k.clone(), base.v.clone(), base.len.clone())
+        rs = running_sum_of(c, lens)
+        kept = torch.full(us + (N,), -7, dtype=torch.int32, device="cuda")
+        ev = torch.full(us, -7, dtype=torch.int32, device="cuda")
+        if decode:
+            vd.vd_append_evict_decode(c, k, v, N, None, oracle.L2, vd.VD_MU_RUNNING, rs, ev, kept)
+        else:
+            vd.vd_append_evict_block(c, k, v, B, N, None, oracle.L2, vd.VD_MU_RUNNING, rs, kept)
+        assert vd.vd_get_device_status() == 0
+        check_running_sum(c, rs)
+        got.append((c.len.clone(), kept, ev) + tuple(
+            t[s, ..., :n, :].view(torch.int16) for t in (c.k, c.v)
+            for s, n in enumerate(c.len.tolist())))
+    assert len(got[0]) == len(got[1])
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
