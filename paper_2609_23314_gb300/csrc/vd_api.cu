@@ -25,9 +25,9 @@ const void* evict_kernel_norm(bool decode, bool holefill, bool fused, bool gener
 const void* small_kernel_l2(bool decode, bool fused);
 const void* small_kernel_dir(bool decode, bool fused);
 const void* small_kernel_norm(bool decode, bool fused);
-const void* resident_kernel_l2(bool decode, bool fused);
-const void* resident_kernel_dir(bool decode, bool fused);
-const void* resident_kernel_norm(bool decode, bool fused);
+const void* resident_kernel_l2(bool decode, bool holefill, bool fused);
+const void* resident_kernel_dir(bool decode, bool holefill, bool fused);
+const void* resident_kernel_norm(bool decode, bool holefill, bool fused);
 const void* score_kernel_l2(bool general);
 const void* score_kernel_dir();
 const void* score_kernel_norm(bool general);
@@ -172,11 +172,11 @@ const void* small_kernel(vd_variant var, bool decode, bool fused) {
   }
 }
 
-const void* resident_kernel(vd_variant var, bool decode, bool fused) {
+const void* resident_kernel(vd_variant var, bool decode, bool holefill, bool fused) {
   switch (var) {
-    case VD_SCORE_L2: return vd::resident_kernel_l2(decode, fused);
-    case VD_SCORE_DIR: return vd::resident_kernel_dir(decode, fused);
-    default: return vd::resident_kernel_norm(decode, fused);
+    case VD_SCORE_L2: return vd::resident_kernel_l2(decode, holefill, fused);
+    case VD_SCORE_DIR: return vd::resident_kernel_dir(decode, holefill, fused);
+    default: return vd::resident_kernel_norm(decode, holefill, fused);
   }
 }
 
@@ -215,11 +215,11 @@ vd_status device_state(DeviceState** out) {
           return VD_ERR_CUDA;
       }
     for (int var = 0; var < 3; ++var)
-      for (int kind = 0; kind < 10; ++kind) {
+      for (int kind = 0; kind < 14; ++kind) {
         const bool dec = (kind & 1) != 0, fus = (kind & 2) != 0;
-        const void* kern = kind >= 8  ? score_kernel((vd_variant)var, kind == 9)
+        const void* kern = kind >= 12 ? score_kernel((vd_variant)var, kind == 13)
                            : kind < 4 ? small_kernel((vd_variant)var, dec, fus)
-                                      : resident_kernel((vd_variant)var, dec, fus);
+                                      : resident_kernel((vd_variant)var, dec, kind >= 8, fus);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  st.smem_optin) != cudaSuccess ||
             cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
@@ -570,7 +570,7 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
   return VD_OK;
 }
 
-// The resident kernel (vd_resident.cuh) takes an ordered eviction whose
+// The resident kernel (vd_resident.cuh) takes an eviction whose
 // clusters all run at once: it is bound by the latency of its phases, so it
 // wins where the streaming kernel has too few rows per SM to hide its own, and
 // loses once several waves of clusters follow one another (288 units of 2176
@@ -586,13 +586,18 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
 // kernel.  us, streaming / resident: d = 64, 340 rows, 320 units 26.8 / 22.4, 4800
 // units 208 / 182; d = 96, 240 rows, 1600 units 105 / 86 (340 rows, two CTAs per
 // SM, 110 / 127); decode, d = 128, 301 rows, 640 units 42.9 / 33.7, 4800 units
-// 197 / 172 (451 rows, one CTA per SM, 249 / 328).  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
+// 197 / 172 (451 rows, one CTA per SM, 249 / 328).  A hole-fill block event moves
+// so few rows that the streaming kernel catches up at 18 MB of scored rows (d =
+// 256, 1128 rows, 16 units 25.3 / 22.6, 32 units 27.6 / 29.7); otherwise the same
+// lines: hole-fill block, d = 128, 2176 rows, 8 units 22.8 / 18.0, 230 rows, 320
+// units 39.1 / 20.1; hole-fill decode, 4097 rows, 8 units 19.2 / 11.0, 201 rows,
+// 4800 units 138 / 86.  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
 // c CTAs (100 + c: with both buffers), for tests.  Returns C, or 0.
 constexpr int kResidentKind = 4;  // and 5: with the running mean
 constexpr int kResidentMinRows = 64;
 
 int resident_plan(const void* kern, long long units, int d, int capacity, bool decode,
-                  bool running, DeviceState& st, size_t* smem_out, bool* both_out) {
+                  bool holefill, bool running, DeviceState& st, size_t* smem_out, bool* both_out) {
   const char* env = std::getenv("VD_RESIDENT");
   const int want = env ? std::atoi(env) : -1;
   if (want == 0 || std::getenv("VD_CLUSTER_SIZE") || capacity > 32768) return 0;
@@ -610,7 +615,7 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
     }
   }
   auto smem_of = [&](int c, bool both) {
-    return vd::resident_layout(capacity, d, c, decode, running, both).total;
+    return vd::resident_layout(capacity, d, c, decode, holefill, running, both).total;
   };
   // units that run at once on clusters of c CTAs
   auto at_once = [&](int c, bool both) -> long long {
@@ -621,7 +626,7 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
   bool both = false;
   if (want > 0) {
     c = want % 100;
-    both = want >= 100;
+    both = want >= 100 && !holefill;
     if (c < 1 || c > vd::kResMaxCluster || at_once(c, both) < 1) c = 0;
   } else {
     const long long room = (decode ? 3LL : 2LL) * st.sms;
@@ -629,8 +634,9 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
       const long long most = std::min<long long>(room / units, capacity / kResidentMinRows);
       for (c = (int)std::max(1LL, std::min(12LL, most)); c >= 1; --c)
         if (at_once(c, false) >= units) break;
-      both = c >= 1 && at_once(c, true) >= units;
+      both = !holefill && c >= 1 && at_once(c, true) >= units;
     }
+    if (holefill && !decode && c > 1 && units * capacity * d * 2 > 18LL << 20) c = 0;
     if (c < 1 && at_once(1, false) >= (decode ? 2LL : 3LL) * st.sms) c = 1;
   }
   const size_t smem = c >= 1 ? smem_of(c, both) : 0;
@@ -750,11 +756,11 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   }
   size_t smem = 0;
   long long solo = 0;
-  if (!score_only && !holefill) {
-    const void* rk = resident_kernel(var, decode, fused);
+  if (!score_only) {
+    const void* rk = resident_kernel(var, decode, holefill, fused);
     bool both = false;
-    a.cluster = resident_plan(rk, units, c->head_dim, c->capacity, decode, mu == VD_MU_RUNNING,
-                              *st, &smem, &both);
+    a.cluster = resident_plan(rk, units, c->head_dim, c->capacity, decode, holefill,
+                              mu == VD_MU_RUNNING, *st, &smem, &both);
     if (a.cluster > 0) {
       const vd::ResidentArgs ra{a, both ? 1 : 0};
       r = launch(rk, units, a.cluster, smem, &ra, s, true);

@@ -1,8 +1,8 @@
-// vd_resident.cuh -- pi_N of Sec. 2.1 Eq. (eviction), ordered layout, with the
-// scored rows of a unit kept in the shared memory of its thread-block cluster.
+// vd_resident.cuh -- pi_N of Sec. 2.1 Eq. (eviction) with the scored rows of a
+// unit kept in the shared memory of its thread-block cluster.
 //
-// For launches of few units, where the streaming kernel (vd_evict.cuh) waits
-// for its own phases: a cluster of C CTAs (any C up to 16) loads a unit's
+// For launches of few or small units, where the streaming kernel (vd_evict.cuh)
+// waits for its own phases: a cluster of C CTAs (any C up to 16) loads a unit's
 // scored rows once.  CTA r holds the rows [r * R, (r + 1) * R) and the mean,
 // the scores, the retired part of the running sum and the compacted rows all
 // come from that copy (the streaming kernel reads the scored tensor twice,
@@ -25,13 +25,15 @@
 //              gather has no order to respect.  The other tensor's slice is
 //              then loaded into the same buffer (it was brought to L2 during
 //              steps 2 to 4), or was loaded with the first one where both
-//              fit, and written after one more barrier.
+//              fit, and written after one more barrier.  Hole-fill layout:
+//              only the movers are copied, from global memory into the holes.
 //
 // What bounds it: the latency of these steps, each of which runs once.  At 8
 // units of 2176 rows, d = 128 (C = 12) a call takes 19.6 us, 29.0 with the
 // streaming kernel; ncu counts half of the warps' stalls as instruction fetch
-// (no loop repeats often enough to stay cached), so loops are kept rolled and
-// 8 warps per CTA beat 16 (17.9 us against 19.6 on one box).  The barriers that
+// (no loop repeats often enough to stay cached).  8 warps per CTA beat 16 (17.9
+// us against 19.6 on one box), and rolling the loops up lost 0.8 us: the loads
+// that an unrolled loop keeps in flight count for more.  The barriers that
 // only order execution are relaxed arrivals: the release form waited 2 to 5 us
 // for the bulk copies in flight.  Recomputed mean at 8 units: 35.0 -> 26.5 us;
 // Dir 35.5 -> 21.8; d = 96 32.9 -> 17.5; decode, 4097 rows 25.5 -> 16.1.
@@ -64,6 +66,8 @@ struct ResSmem {
   double snew[256];  // running mode: the running sum plus the appended rows
   unsigned long long bar[kResChunks + 1];  // scored tensor's chunks, other tensor
   unsigned long long best[kResMaxCluster];  // decode: every CTA's minimum (pushed by it)
+  int best_slot[kResMaxCluster];            // hole-fill decode: its slot (pushed)
+  int wslot[kWarps];
   uint32_t kmin[kResMaxCluster];  // every CTA's smallest and largest key (pushed)
   uint32_t kmax[kResMaxCluster];
   unsigned long long wbest[kWarps];
@@ -85,21 +89,23 @@ __host__ __device__ inline int resident_rows(int n, int c) {
 }
 
 struct ResLayout {
-  size_t keys, list, buf, obuf, total;
+  size_t keys, list, pairs, buf, obuf, total;
 };
 
 // The keys' region also holds resident_sum's partials, before the keys are
-// written and after they are last read.  Decode keeps no keys, and sums rows
+// written.  Decode keeps no keys, and sums rows
 // only where the mean is recomputed.
 __host__ __device__ inline ResLayout resident_layout(int capacity, int d, int cluster, bool decode,
-                                                     bool running, bool both) {
+                                                     bool holefill, bool running, bool both) {
   const size_t rcap = (size_t)resident_rows(capacity, cluster);
   const size_t keys = decode ? 0 : rcap * (size_t)cluster * 4;
-  const size_t scratch = decode && running ? 0 : (size_t)(d < 32 ? 32 : d) * kWarps * 8;
+  const size_t scratch = decode && running ? 0 : (size_t)d * kWarps * 8;
   ResLayout l;
   l.keys = (sizeof(ResSmem) + 127) & ~(size_t)127;
   l.list = l.keys + (keys > scratch ? keys : scratch);
-  l.buf = (l.list + (decode ? 0 : rcap * 2) + 127) & ~(size_t)127;
+  l.pairs = (l.list + (decode ? 0 : rcap * 2) + 3) & ~(size_t)3;
+  // hole-fill: at most half of the rows are holes, and as many movers
+  l.buf = (l.pairs + (decode || !holefill ? 0 : (size_t)capacity * 2 + 4) + 127) & ~(size_t)127;
   const size_t bytes = (rcap * (size_t)d * 2 + 127) & ~(size_t)127;
   l.obuf = both ? l.buf + bytes : l.buf;
   l.total = l.obuf + bytes;
@@ -359,30 +365,19 @@ __device__ __forceinline__ void resident_score_general(uint32_t buf, int ca, int
   }
 }
 
-// The N-th largest of keys[0, n) (all in this CTA's shared memory), how many
+// The N-th largest of a unit's keys (all in this CTA's reach), how many
 // keys equal to it are kept, and how many there are.  [kmin, kmax] spans the
 // keys.  A pass spreads the keys of the current range over 1024 buckets of
 // equal width and keeps the bucket that holds the threshold; at most 256 keys
 // in it are ranked directly.  The range shrinks 1024-fold per pass, so there
 // are at most four (fp32 keys of one unit differ in a few high bits: one pass
 // resolves all but heavily tied caches).
-__device__ __forceinline__ Selection resident_select(const uint32_t* keys, int n, int N,
-                                                     uint32_t kmin, uint32_t kmax, ResSmem& S) {
+// for_keys(use) calls use(key) for every key, spread over the threads.
+template <class ForKeys>
+__device__ __forceinline__ Selection resident_select(ForKeys for_keys, int N, uint32_t kmin,
+                                                     uint32_t kmax, ResSmem& S) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint32_t* hist = reinterpret_cast<uint32_t*>(S.mu);
-  // every key in turn, four per load
-  auto for_keys = [&](auto use) {
-    const int nv = n >> 2;
-#pragma unroll 2
-    for (int i = tid; i < nv; i += kThreads) {
-      const uint4 k = reinterpret_cast<const uint4*>(keys)[i];
-      use(k.x);
-      use(k.y);
-      use(k.z);
-      use(k.w);
-    }
-    if (tid < (n & 3)) use(keys[4 * nv + tid]);
-  };
   int need = N;
   for (;;) {
     const uint32_t range = kmax - kmin;
@@ -462,11 +457,12 @@ __device__ __forceinline__ Selection resident_select(const uint32_t* keys, int n
   }
 }
 
-// VAR: 0 L2, 1 Dir, 2 Norm.  DECODE: one token is evicted (arg-min).  FUSED:
-// rows at or above len come from the caller's staging buffers.  Same
-// arguments, validation, outputs and status codes as evict_kernel in the
-// ordered layout.
-template <int VAR, bool DECODE, bool FUSED>
+// VAR: 0 L2, 1 Dir, 2 Norm.  DECODE: one token is evicted (arg-min).  HF: the
+// hole-fill layout (ties by token position; only the kept rows at or above the
+// budget move, from where they are in global memory: the other tensor is not
+// loaded).  FUSED: rows at or above len come from the caller's staging buffers.
+// Same arguments, validation, outputs and status codes as evict_kernel.
+template <int VAR, bool DECODE, bool HF, bool FUSED>
 __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const ResidentArgs ra) {
   const EvictArgs& a = ra.e;
   // launched as a programmatic dependent: lets the next kernel be scheduled,
@@ -482,10 +478,12 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
   }
   grid_dependency_wait();
   const int C = a.cluster, d = a.d, d8 = d >> 3, lpr = a.lpr, cap = a.capacity;
-  const ResLayout L = resident_layout(cap, d, C, DECODE, a.mu_running != 0, ra.both != 0);
+  const ResLayout L = resident_layout(cap, d, C, DECODE, HF, a.mu_running != 0, ra.both != 0);
   uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + L.keys);
   float* scratch = reinterpret_cast<float*>(smem_raw + L.keys);
   uint16_t* list = reinterpret_cast<uint16_t*>(smem_raw + L.list);
+  uint16_t* holes = reinterpret_cast<uint16_t*>(smem_raw + L.pairs);
+  uint16_t* movers = holes + (cap >> 1);
   const uint32_t sbuf = smem_addr(smem_raw + L.buf), obuf = smem_addr(smem_raw + L.obuf);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned rank = C > 1 ? cluster_ctarank() : 0u;
@@ -515,6 +513,11 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
   uint16_t* ob = a.score_k ? vb : kb;
   const uint16_t* snu = a.score_k ? knu : vnu;
   const uint16_t* onu = a.score_k ? vnu : knu;
+  // hole-fill layout: token positions (rows at or above first_new are the
+  // appended ones, numbered from pos_new)
+  int32_t* posu = HF ? a.pos + (size_t)u * cap : nullptr;
+  const int pnew = HF ? a.pos_new[seq] : 0;
+  auto pos_of = [&](int r) -> int { return r < first_new ? posu[r] : pnew + (r - first_new); };
 
   if (n <= Nb) {
     // ---- nothing to evict: append (fused), identity outputs, running sum ---
@@ -523,6 +526,8 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
       copy_new_rows(kb, vb, knu + (size_t)i0 * d, vnu + (size_t)i0 * d, d, 0, 2 * d8, len0 + i0,
                     i1 - i0);
     }
+    if (HF && rank == 0)
+      for (int r = max(first_new, 0) + tid; r < n; r += kThreads) posu[r] = pnew + (r - first_new);
     if (a.kept_out)
       for (int i = (int)rank * kThreads + tid; i < a.N; i += C * kThreads)
         a.kept_out[(size_t)u * a.N + i] = i < n ? i : -1;
@@ -566,9 +571,9 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
   if (tid == 0) {
     for (int i = 0; i < nch; ++i)
       load_rows(sbuf, sb, snu, i * rch, min(R, (i + 1) * rch), bar_s + 8u * (uint32_t)i);
-    if (ra.both)
+    if (!HF && ra.both)
       load_rows(obuf, ob, onu, 0, R, bar_o);
-    else if (!DECODE && fs > 0)  // on its way to L2 while the scores and the select run
+    else if (!HF && !DECODE && fs > 0)  // on its way to L2 while the scores and the select run
       bulk_prefetch_l2(ob + (size_t)r0 * d, (uint32_t)(fs * row_bytes));
   }
   __syncthreads();
@@ -650,7 +655,8 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
   const bool disp = VAR == 0 && !DECODE && a.disp_out != nullptr;
   float ds_hi = 0.f, ds_lo = 0.f, dq_hi = 0.f, dq_lo = 0.f;
   unsigned long long best = ~0ull;
-  uint32_t kmin = 0xffffffffu, kmax = 0u;
+  uint32_t kmin = 0xffffffffu, kmax = 0u;  // (hole-fill decode: kmin is the minimum's key)
+  int best_slot = -1;
   {
     float* sc_out = a.scores_out ? a.scores_out + (size_t)u * cap + r0 : nullptr;
     const float* wu = !DECODE && a.weights ? a.weights + (size_t)u * cap + r0 : nullptr;
@@ -673,10 +679,15 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
         if (bad) record_status(a.status, kStNonfinite);
       }
       if (sc_out) sc_out[j] = s;
-      if (DECODE) {
+      if (DECODE && !HF) {
         const unsigned long long pk = ((unsigned long long)key << 32) |
                                       (unsigned long long)(0xffffffffu - (unsigned)(r0 + j));
         best = pk < best ? pk : best;
+      } else if (DECODE) {  // positions are read only to settle an exact tie
+        if (key < kmin || best_slot < 0 || (key == kmin && pos_of(r0 + j) > pos_of(best_slot))) {
+          kmin = key;
+          best_slot = r0 + j;
+        }
       } else {
         keys[r0 + j] = key;
         kmin = min(kmin, key);
@@ -699,27 +710,60 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
 
   // ---- 4. exchange, select, kept list --------------------------------------
   int kept_off = 0, nk = 0, e_first = n;  // block: this slice's kept rows; decode: the evicted slot
+  int nhole = 0;                          // hole-fill block: rows that move
+  uint32_t tkey = 0u;                     // hole-fill block: a row with key > tkey is kept
   if (DECODE) {
-    best = warp_min_u64(best);
+    if (HF) {
+      if (best_slot >= 0)
+        best = ((unsigned long long)kmin << 32) |
+               (unsigned long long)(0xffffffffu - (unsigned)pos_of(best_slot));
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(kFull, best, off);
+        const int os = __shfl_xor_sync(kFull, best_slot, off);
+        if (o < best) {
+          best = o;
+          best_slot = os;
+        }
+      }
+      if (lane == 0) S.wslot[warp] = best_slot;
+    } else {
+      best = warp_min_u64(best);
+    }
     if (lane == 0) S.wbest[warp] = best;
     __syncthreads();
     if (!met) cluster_wait();
     if (tid < C) {
       unsigned long long b = ~0ull;
+      int bs = -1;
 #pragma unroll
-      for (int w = 0; w < kWarps; ++w) b = S.wbest[w] < b ? S.wbest[w] : b;
-      const uint32_t at = smem_addr(&S.best[rank]);
-      if (C > 1) st_cluster_u64(mapa(at, (unsigned)tid), b);
-      else S.best[0] = b;
+      for (int w = 0; w < kWarps; ++w) {
+        if (HF && S.wbest[w] < b) bs = S.wslot[w];
+        b = S.wbest[w] < b ? S.wbest[w] : b;
+      }
+      if (C > 1) {
+        st_cluster_u64(mapa(smem_addr(&S.best[rank]), (unsigned)tid), b);
+        if (HF) st_cluster_u32(mapa(smem_addr(&S.best_slot[rank]), (unsigned)tid), (uint32_t)bs);
+      } else {
+        S.best[0] = b;
+        S.best_slot[0] = bs;
+      }
     }
-    if (ra.both) mbar_wait(bar_o, 0u, a.status);
+    if (!HF && ra.both) mbar_wait(bar_o, 0u, a.status);
     if (C > 1) cluster_sync(); else __syncthreads();
-    const unsigned long long b = warp_min_u64(lane < C ? S.best[lane] : ~0ull);
-    e_first = (int)(0xffffffffu - (unsigned)(b & 0xffffffffull));
+    const unsigned long long mine = lane < C ? S.best[lane] : ~0ull;
+    const unsigned long long b = warp_min_u64(mine);
+    if (HF) {  // positions are distinct: one CTA has it
+      const unsigned who = __ballot_sync(kFull, mine == b && lane < C);
+      e_first = max(0, min(S.best_slot[__ffs(who) - 1], n - 1));
+    } else {
+      e_first = (int)(0xffffffffu - (unsigned)(b & 0xffffffffull));
+    }
     if (a.evicted_out && rank == 0 && tid == 0) a.evicted_out[u] = e_first;
     if (a.kept_out)
       for (int i = (int)rank * kThreads + tid; i < a.N; i += C * kThreads)
-        a.kept_out[(size_t)u * a.N + i] = i < Nb ? (i < e_first ? i : i + 1) : -1;
+        a.kept_out[(size_t)u * a.N + i] =
+            i >= Nb ? -1 : HF ? (i == e_first ? n - 1 : i) : i < e_first ? i : i + 1;
   } else {
     kmin = __reduce_min_sync(kFull, kmin);
     kmax = __reduce_max_sync(kFull, kmax);
@@ -783,11 +827,45 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
         }
       }
     }
-    if (ra.both) mbar_wait(bar_o, 0u, a.status);
+    if (!HF && ra.both) mbar_wait(bar_o, 0u, a.status);
     if (C > 1) cluster_sync(); else __syncthreads();
     kmin = __reduce_min_sync(kFull, lane < C ? S.kmin[lane] : 0xffffffffu);
     kmax = __reduce_max_sync(kFull, lane < C ? S.kmax[lane] : 0u);
-    const Selection sel = resident_select(keys, n, Nb, kmin, kmax, S);
+    Selection sel = resident_select(
+        [&](auto use) {  // four keys per load
+          const int nv = n >> 2;
+#pragma unroll 2
+          for (int i = tid; i < nv; i += kThreads) {
+            const uint4 k = reinterpret_cast<const uint4*>(keys)[i];
+            use(k.x);
+            use(k.y);
+            use(k.z);
+            use(k.w);
+          }
+          if (tid < (n & 3)) use(keys[4 * nv + tid]);
+        },
+        Nb, kmin, kmax, S);
+    if (HF) {
+      // a kept row is one with key > t from here on: the surviving ties are
+      // the lowest positions, found by a second select over the complemented
+      // positions of the tied rows, whose keys this CTA's copy then raises
+      // (t >= 1 where every tie survives: a row with a lower key goes)
+      if (sel.cnt_eq > sel.keep_eq) {
+        const uint32_t t = sel.t;
+        const Selection s2 = resident_select(
+            [&](auto use) {
+              for (int j = tid; j < n; j += kThreads)
+                if (keys[j] == t) use(~(uint32_t)pos_of(j));
+            },
+            sel.keep_eq, 0u, 0xffffffffu, S);
+        for (int j = tid; j < n; j += kThreads)
+          if (keys[j] == t && ~(uint32_t)pos_of(j) >= s2.t) keys[j] = t + 1u;
+        __syncthreads();
+      } else {
+        sel.t -= 1u;
+      }
+      sel.keep_eq = 0;
+    }
     if (VAR == 0 && disp && rank == 0 && tid == 0) {
       double s1 = 0.0, s2 = 0.0;
       const uint32_t base = smem_addr(&S.disp[0]);
@@ -805,6 +883,7 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
     // kept list: counts of keys > t (low half) and == t (high half) before
     // this slice, and before this thread's rows of it; ties go to the lower slot
     const uint32_t t = sel.t;
+    tkey = t;
     const int q = sel.keep_eq;
     auto count = [&](uint32_t key) { return (key > t ? 1u : 0u) + (key == t ? 0x10000u : 0u); };
     uint32_t before = 0u, mine = 0u;
@@ -845,6 +924,40 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
       if ((unsigned)pos < (unsigned)R) list[pos] = (uint16_t)j;
       else record_status(a.status, kStInternal);  // never for a consistent selection
     }
+    if (HF) {
+      // the evicted slots below the budget and the kept ones at or above it,
+      // ascending (every CTA lists them all), by contiguous runs of slots
+      auto kind = [&](int r) {  // hole: low half, mover: high half
+        const bool kp = keys[r] > t;
+        return r < Nb ? (kp ? 0u : 1u) : (kp ? 0x10000u : 0u);
+      };
+      const int run = (n + kThreads - 1) / kThreads;
+      const int x = min(n, tid * run), y = min(n, x + run);
+      uint32_t own = 0u;
+      for (int r = x; r < y; ++r) own += kind(r);
+      uint32_t sum = own;
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const uint32_t z = __shfl_up_sync(kFull, sum, off);
+        if (lane >= off) sum += z;
+      }
+      if (lane == 31) S.wslot[warp] = (int)sum;
+      __syncthreads();
+      uint32_t at2 = sum - own, all = 0u;
+#pragma unroll
+      for (int w = 0; w < kWarps; ++w) {
+        all += (uint32_t)S.wslot[w];
+        if (w < warp) at2 += (uint32_t)S.wslot[w];
+      }
+      nhole = min((int)(all & 0xffffu), cap >> 1);
+      if ((all & 0xffffu) != (all >> 16) && tid == 0) record_status(a.status, kStInternal);
+      for (int r = x; r < y; ++r) {
+        const uint32_t kd = kind(r);
+        if ((kd & 1u) && (int)(at2 & 0xffffu) < nhole) holes[at2 & 0xffffu] = (uint16_t)r;
+        if ((kd >> 16) && (int)(at2 >> 16) < nhole) movers[at2 >> 16] = (uint16_t)r;
+        at2 += kd;
+      }
+    }
     __syncthreads();
   }
 
@@ -867,26 +980,90 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
             (uint32_t)reinterpret_cast<const uint16_t*>(smem_raw + L.buf)[j * d + c] << 16);
         ff_accumulate(hi, lo, i < nnew ? x : -x);
       }
-      scratch[part * d + c] = hi;
-      scratch[kThreads + part * d + c] = lo;
+      S.mu[part * d + c] = hi;  // the histogram's memory is free again
+      S.mulo[part * d + c] = lo;
     }
     __syncthreads();
     if (tid < d) {
       ff t{0.f, 0.f};
 #pragma unroll 1
       for (int m = 0; m < parts; ++m)
-        t = ff_add(t, ff{scratch[m * d + tid], scratch[kThreads + m * d + tid]});
+        t = ff_add(t, ff{S.mu[m * d + tid], S.mulo[m * d + tid]});
       S.acc_hi[tid] = t.hi;
       S.acc_lo[tid] = t.lo;
     }
     if (C > 1) cluster_arrive(); else __syncthreads();
   }
-  if (!DECODE && a.kept_out) {
+  if (!DECODE && !HF && a.kept_out) {
     int32_t* ko = a.kept_out + (size_t)u * a.N;
     for (int i = tid; i < nk; i += kThreads)
       if (kept_off + i < a.N) ko[kept_off + i] = r0 + (int)list[i];
     if (rank == 0)
       for (int i = Nb + tid; i < a.N; i += kThreads) ko[i] = -1;
+  }
+
+  if constexpr (HF) {
+    // ---- 6. hole-fill: movers into holes, from where they are -------------
+    // Every source lies at or above the budget and every destination below it;
+    // the holes' old rows are in shared memory since before the exchange.
+    const int ci = lane & (lpr - 1), g = tid / lpr, ng = kThreads / lpr;
+    auto copy_row = [&](int item, int src, int dst) {  // item & 1: K or V
+      const uint16_t* from = src >= first_stage
+                                 ? ((item & 1) ? vnu : knu) + (size_t)(src - first_stage) * d
+                                 : ((item & 1) ? vb : kb) + (size_t)src * d;
+      st16(((item & 1) ? vb : kb) + (size_t)dst * d + ci * 8, ld_cg16(from + ci * 8));
+    };
+    if (DECODE) {
+      if (rsu && e_first >= r0 && e_first < r1 && tid < d) {
+        const uint16_t* row =
+            reinterpret_cast<const uint16_t*>(smem_raw + L.buf) + (size_t)(e_first - r0) * d;
+        rsu[tid] = S.snew[tid] - (double)__uint_as_float((uint32_t)row[tid] << 16);
+      }
+      if (rank == 0 && e_first < Nb) {
+        for (int it = g; it < 2 && ci < d8; it += ng) copy_row(it, n - 1, e_first);
+        if (tid == 0) posu[e_first] = pos_of(n - 1);
+      }
+      return;
+    }
+    if (C > 1 && !exchange) cluster_arrive_relaxed();
+    const int mine = nhole > (int)rank ? (nhole - (int)rank + C - 1) / C : 0;
+    if (ci < d8) {
+      for (int it = g; it < 2 * mine; it += ng) {  // pairs rank, rank + C, ...
+        const int i = (int)rank + (it >> 1) * C;
+        copy_row(it, movers[i], holes[i]);
+      }
+      // fused append: kept new rows below the budget into their own slots
+      if (FUSED)
+        for (int it = g;; it += ng) {
+          const int r = first_stage + (int)rank + (it >> 1) * C;
+          if (r >= Nb) break;
+          if (keys[r] > tkey) copy_row(it, r, r);
+        }
+    }
+    if (a.kept_out) {
+      int32_t* ko = a.kept_out + (size_t)u * a.N;
+      for (int r = (int)rank * kThreads + tid; r < a.N; r += C * kThreads)
+        if (r >= Nb || keys[r] > tkey) ko[r] = r < Nb ? r : -1;
+      for (int i = tid; i < mine; i += kThreads) ko[holes[rank + i * C]] = movers[rank + i * C];
+    }
+    if (C > 1) cluster_wait();  // every CTA is done with the positions, and with its partial sums
+    for (int r = max(first_new, 0) + (int)rank * kThreads + tid; r < Nb; r += C * kThreads)
+      if (keys[r] > tkey) posu[r] = pnew + (r - first_new);
+    for (int i = tid; i < mine; i += kThreads)
+      posu[holes[rank + i * C]] = pos_of(movers[rank + i * C]);
+    if (exchange) {
+      const int c = (int)((unsigned)d * rank / (unsigned)C) + tid;
+      if (c < (int)((unsigned)d * (rank + 1) / (unsigned)C)) {
+        const ff t = C > 1 ? resident_gather(c, C, S) : ff{S.acc_hi[c], S.acc_lo[c]};
+        const double base = VAR != 2 ? S.snew[c] : rsu[c];
+        rsu[c] = base + (double)t.hi + (double)t.lo;
+      }
+      if (C > 1) {  // peers have read this CTA's partial results
+        cluster_arrive_relaxed();
+        cluster_wait();
+      }
+    }
+    return;
   }
 
   // ---- 6. kept rows to their slots -----------------------------------------

@@ -4,12 +4,17 @@
 
 namespace vd {
 
-const void* resident_kernel_norm(bool decode, bool fused) {
-  if (decode)
-    return fused ? reinterpret_cast<const void*>(&resident_evict_kernel<2, true, true>)
-                 : reinterpret_cast<const void*>(&resident_evict_kernel<2, true, false>);
-  return fused ? reinterpret_cast<const void*>(&resident_evict_kernel<2, false, true>)
-               : reinterpret_cast<const void*>(&resident_evict_kernel<2, false, false>);
+const void* resident_kernel_norm(bool decode, bool holefill, bool fused) {
+  const void* k[2][2][2] = {
+      {{reinterpret_cast<const void*>(&resident_evict_kernel<2, false, false, false>),
+        reinterpret_cast<const void*>(&resident_evict_kernel<2, false, false, true>)},
+       {reinterpret_cast<const void*>(&resident_evict_kernel<2, false, true, false>),
+        reinterpret_cast<const void*>(&resident_evict_kernel<2, false, true, true>)}},
+      {{reinterpret_cast<const void*>(&resident_evict_kernel<2, true, false, false>),
+        reinterpret_cast<const void*>(&resident_evict_kernel<2, true, false, true>)},
+       {reinterpret_cast<const void*>(&resident_evict_kernel<2, true, true, false>),
+        reinterpret_cast<const void*>(&resident_evict_kernel<2, true, true, true>)}}};
+  return k[decode][holefill][fused];
 }
 
 }  // namespace vd

@@ -46,6 +46,7 @@ def make(n_seq, L, H, cap, d, seed, edit=None):
 
 
 def step(force, k, v, lens, N, B, var, mu, decode, fused, budgets, options, monkeypatch):
+    # (options["pos"]: hole-fill layout, positions of the cached rows)
     """One event of the cache k, v (lens rows each, the last B of them new)
     under VD_RESIDENT=force; every output, the cache and the status."""
     monkeypatch.setenv("VD_RESIDENT", str(force))
@@ -78,7 +79,23 @@ def step(force, k, v, lens, N, B, var, mu, decode, fused, budgets, options, monk
     if options.get("attn"):
         g = torch.Generator(device="cuda").manual_seed(3)
         attn = torch.rand(us + (cap,), generator=g, device="cuda") * 0.02
-    if decode:
+    pos = options["pos"].clone() if "pos" in options else None
+    if pos is not None:
+        first = torch.tensor([10 ** 6 + 1000 * s for s in range(n_seq)], dtype=torch.int32,
+                             device="cuda")
+        hole = dict(pos=pos, pos_first_new=first)
+        if decode and fused:
+            vd.vd_append_evict_decode(cache, *new, N, n_dev, var, mu, rs, ev, kept, sc, **hole)
+        elif decode:
+            vd.vd_evict_decode_holefill(cache, N, pos, first, n_dev, var, mu, rs, ev, kept, sc)
+        elif fused:
+            vd.vd_append_evict_block(cache, *new, B, N, n_dev, var, mu, rs, kept, sc, **hole)
+        else:
+            vd.vd_evict_block_holefill(cache, N, pos, first, n_dev, B, var, mu, rs, kept, sc)
+        for s, m in enumerate(cache.len.tolist()):
+            pos[s, ..., m:] = 0  # unspecified there
+        sg = pos.float()
+    elif decode:
         if fused:
             vd.vd_append_evict_decode(cache, *new, N, n_dev, var, mu, rs, ev, kept, sc)
         else:
@@ -109,7 +126,9 @@ def compare(forces, k, v, lens, N, B, var, mu, decode, fused, monkeypatch, budge
         assert torch.equal(got[3], want[3]), force
         assert torch.equal(got[4] == -3.0, want[4] == -3.0)
         torch.testing.assert_close(got[4], want[4], rtol=score_rtol, atol=0, equal_nan=True)
-        if got[5] is not None:
+        if options and "pos" in options:
+            assert torch.equal(got[5], want[5]), force
+        elif got[5] is not None:
             torch.testing.assert_close(got[5], want[5], rtol=1e-6, atol=0, equal_nan=True)
         for s, n in enumerate(want[0].len.tolist()):
             for a, b in ((got[0].k, want[0].k), (got[0].v, want[0].v)):
@@ -179,6 +198,51 @@ def test_ties_and_nonfinite(kind, decode, monkeypatch):
     k, v = make(1, 1, 2, cap, 64, seed=9, edit=edit)
     for var, mu in ((NORM, REC), (L2, REC)):
         compare((1, 2, 9, 104), k, v, [cap], cap - B, B, var, mu, decode, False, monkeypatch)
+
+
+def shuffled_positions(n_seq, L, H, cap, seed):
+    """Distinct positions in no slot order, as after many hole-fill events."""
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    p = torch.rand(n_seq, L, H, cap, generator=g, device="cuda").argsort(-1)
+    return (3 * p).to(torch.int32)
+
+
+@pytest.mark.parametrize("var,mu,decode,fused", FORMS)
+def test_holefill_forms(var, mu, decode, fused, monkeypatch):
+    """Hole-fill layout: budgets above the cached rows (new rows kept in
+    place), below them (movers from the cache too), and equal; positions that
+    do not follow the slots; duplicates, so that positions decide ties."""
+    def edit(k, v):
+        v[:, :, :, 1::7] = v[:, :, :, :1]
+    B = 1 if decode else 37
+    for d, cap, forces in ((128, 333, (1, 3, 8)), (96, 300, (2, 7)), (8, 50, (1, 16)),
+                           (256, 131, (4, 11))):
+        N = cap - B
+        lens = [cap, N + 1, N] if not decode else [cap, N, cap - 2]
+        lens = [max(n, B) for n in lens]
+        budgets = [N, max(1, N - 9), N] if not decode else [N, N, N - 2]
+        k, v = make(3, 1, 2, cap, d, seed=d + B, edit=edit)
+        compare(forces, k, v, lens, N, B, var, mu, decode, fused, monkeypatch, budgets,
+                dict(pos=shuffled_positions(3, 1, 2, cap, d)))
+
+
+@pytest.mark.parametrize("kind", ["all_equal", "many_equal", "nan"])
+@pytest.mark.parametrize("decode", [False, True])
+def test_holefill_ties(kind, decode, monkeypatch):
+    def edit(k, v):
+        n = v.shape[3]
+        if kind == "all_equal":
+            v[:] = 1.5
+        elif kind == "many_equal":
+            v[:, :, :, n // 4:] = v[:, :, :, :1]
+        else:
+            v[:, :, :, 5, 3] = float("nan")
+    cap = 1300
+    B = 1 if decode else 300
+    k, v = make(1, 1, 2, cap, 64, seed=9, edit=edit)
+    for var, N in ((NORM, cap - B), (L2, cap - B)) + (() if decode else ((NORM, 900),)):
+        compare((1, 2, 9), k, v, [cap], N, B, var, REC, decode, False, monkeypatch,
+                options=dict(pos=shuffled_positions(1, 1, 2, cap, 4)))
 
 
 @pytest.mark.parametrize("N", [1, 2, 255, 1023])
