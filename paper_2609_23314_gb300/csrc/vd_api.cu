@@ -501,17 +501,17 @@ int cached_cluster(const void* kern, long long units, int d, int capacity, int k
 // The short-cache kernel (vd_small.cuh) takes a block or decode event when
 // the unit's K and V rows fit in shared memory with room to spare
 // (capacity * head_dim * 4 bytes <= kSmallRowBytes, capacity <=
-// vd::kSmallMaxRows) and no scoring option, hole-fill layout or forced cluster
-// size (VD_CLUSTER_SIZE) is asked for.  It sets the lengths itself where a
+// vd::kSmallMaxRows) and no sigma, hole-fill layout or forced cluster size
+// (VD_CLUSTER_SIZE) is asked for.  It sets the lengths itself where a
 // sequence's units fit in one cluster (<= 16) and the launch is at most one CTA
 // per SM (60 units of 160 rows 9.5 us; 200 units 13.2, and 12.9 without).
 // VD_SMALL_PATH=0 turns it off.  The choice depends on the shape only, so the
 // fused and two-call forms, block and decode, take the same kernel.
 constexpr size_t kSmallRowBytes = 64 * 1024;
 
-bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* weights,
-               const float* disp_out, int score_k, const DeviceState& st) {
-  if (score_only || holefill || weights || disp_out || score_k) return false;
+bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* disp_out,
+               const DeviceState& st) {
+  if (score_only || holefill || disp_out) return false;
   const char* off = std::getenv("VD_SMALL_PATH");
   if ((off && std::atoi(off) == 0) || std::getenv("VD_CLUSTER_SIZE")) return false;
   if (c->capacity > vd::kSmallMaxRows) return false;
@@ -739,7 +739,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     }
     return VD_OK;
   };
-  if (use_small(c, score_only, holefill, weights, disp_out, score_k, *st)) {
+  if (use_small(c, score_only, holefill, disp_out, *st)) {
     const void* sk = small_kernel(var, decode, fused);
     const size_t ssmem = vd::small_layout(c->capacity, c->head_dim).total;
     // few units: n_seq clusters of units_per_seq CTAs (one CTA per unit), which

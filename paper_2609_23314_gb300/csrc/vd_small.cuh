@@ -32,9 +32,8 @@
 // 128, 128 rows, 320 units 23.7 / 15.7, 1600 units 64 / 42, 4800 units 179 / 108;
 // decode, 101 rows, 1600 units 50 / 29.
 //
-// Same validation, outputs and status codes as the fused kernel; no
-// hole-fill layout, attention weights, sigma or key-side rule (those calls
-// take the fused kernel).
+// Same validation, outputs and status codes as the fused kernel; no hole-fill
+// layout and no sigma (those calls take the other kernels).
 #pragma once
 
 #include <cstdint>
@@ -145,10 +144,12 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
   const int n = len0 + (FUSED ? a.B : 0);
   const int Nb = unit_ok ? (a.N_dev ? a.N_dev[seq] : a.N) : 0;
   const size_t ubase = (size_t)u * cap * d;
-  uint16_t* kb = a.k + ubase;
-  uint16_t* vb = a.v + ubase;
-  const uint16_t* knu = FUSED ? a.k_new + (size_t)u * a.B * d : nullptr;
-  const uint16_t* vnu = FUSED ? a.v_new + (size_t)u * a.B * d : nullptr;
+  // "V" is the scored tensor below: K for the key-side rule (the two are
+  // otherwise treated alike)
+  uint16_t* kb = (a.score_k ? a.v : a.k) + ubase;
+  uint16_t* vb = (a.score_k ? a.k : a.v) + ubase;
+  const uint16_t* knu = FUSED ? (a.score_k ? a.v_new : a.k_new) + (size_t)u * a.B * d : nullptr;
+  const uint16_t* vnu = FUSED ? (a.score_k ? a.k_new : a.v_new) + (size_t)u * a.B * d : nullptr;
 
   // ---- validation: the same per-sequence checks as the fused kernel -------
   bool ok = unit_ok;
@@ -236,10 +237,18 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
       }
       // ---- 2. scores: lpr lanes per row, one 16-byte chunk each ----------
       float* sc_out = a.scores_out ? a.scores_out + (size_t)u * cap : nullptr;
+      const float* wu = !DECODE && a.weights ? a.weights + (size_t)u * cap : nullptr;
       resident_score_general<VAR>(vs_a, 0, n, d, a.lpr, S, [&](int j, float sc) {
         bool bad;
-        keys[j] = score_key(sc, bad);
+        uint32_t key = score_key(sc, bad);
         if (bad) record_status(a.status, kStNonfinite);
+        if (!DECODE && wu) {  // a_j / (1 - a_j) * s_j (the FastCAOTE form of App. A)
+          const float w = wu[j];
+          sc = key_score(key) * ((w >= 0.f && w < 1.f) ? w / (1.f - w) : __int_as_float(0x7fc00000));
+          key = score_key(sc, bad);
+          if (bad) record_status(a.status, kStNonfinite);
+        }
+        keys[j] = key;
         if (sc_out) sc_out[j] = sc;
       });
       __syncthreads();

@@ -284,3 +284,52 @@ def test_many_units_match_the_streaming_kernel(decode, shape, monkeypatch):
     assert len(got[0]) == len(got[1])
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
+@pytest.mark.parametrize("mu", MUS, ids=MU_IDS)
+@pytest.mark.parametrize("keys,attn", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("fused", [False, True])
+def test_scoring_options_match_the_streaming_kernel(var, mu, keys, attn, fused, monkeypatch):
+    """The key-side rule and attention weights (one weight of 1: a NaN score),
+    with and without the cluster that sets the lengths."""
+    monkeypatch.setenv("VD_RESIDENT", "0")
+    for n_seq, H, d, cap, B in ((2, 3, 64, 150, 40), (9, 18, 24, 60, 11)):
+        N = cap - B
+        lens = [N - (s == 1) * B for s in range(n_seq)]
+        base = filled_cache(n_seq, 1, H, cap, d, lens, seed=cap)
+        us = base.unit_shape()
+        k, v = wl.TokenStream("gauss_outlier", base.units, d, seed=5).next(B)
+        k, v = k.view(us + (B, d)).contiguous(), v.view(us + (B, d)).contiguous()
+        w = None
+        if attn:
+            w = torch.rand(us + (cap,), generator=torch.Generator("cuda").manual_seed(2),
+                           device="cuda") * 0.1
+            w[0, 0, 0, 3] = 1.0
+        got = []
+        for small in ("1", "0"):
+            monkeypatch.setenv("VD_SMALL_PATH", small)
+            c = vd.Cache(base.k.clone(), base.v.clone(), base.len.clone())
+            rs = torch.zeros(us + (d,), dtype=torch.float64, device="cuda") if mu else None
+            if mu:
+                vd.vd_running_sum_init_ex(c, keys, rs)
+            kept = torch.full(us + (N,), -7, dtype=torch.int32, device="cuda")
+            sc = torch.full(us + (cap,), -3.0, device="cuda")
+            if fused:
+                vd.vd_append_evict_block_ex(c, k, v, B, N, None, var, mu, rs, keys, w, kept, sc)
+            else:
+                vd.vd_append(c, k, v, B)
+                vd.vd_evict_block_ex(c, N, None, B, var, mu, rs, keys, w, kept, sc)
+            got.append((vd.vd_get_device_status(), c, rs, kept, sc))
+        (s0, c0, r0, k0, x0), (s1, c1, r1, k1, x1) = got
+        assert s0 == s1 == (4 if attn else 0)
+        assert torch.equal(c0.len, c1.len) and torch.equal(k0, k1)
+        # the L2 and Norm scores of d = 64 add their lanes in another order here
+        torch.testing.assert_close(x0, x1, rtol=2e-6, atol=0, equal_nan=True)
+        for s, n in enumerate(c0.len.tolist()):
+            for a, b in ((c0.k, c1.k), (c0.v, c1.v)):
+                assert torch.equal(a[s, ..., :n, :].view(torch.int16),
+                                   b[s, ..., :n, :].view(torch.int16))
+        if mu:
+            scale = units_view(c0.k if keys else c0.v).float().abs().sum(dim=1).max().item()
+            assert torch.max(torch.abs(r0 - r1)).item() <= 1e-12 * scale
