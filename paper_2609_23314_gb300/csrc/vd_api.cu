@@ -720,6 +720,8 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   a.k_new = static_cast<const uint16_t*>(k_new);
   a.v_new = static_cast<const uint16_t*>(v_new);
   a.unit_base = 0;
+  a.wait_first = 1;
+  a.let_next = score_only ? 0 : 1;
   // the eviction's length update, a programmatic dependent of it
   auto clamp_lengths = [&]() -> vd_status {
     cudaLaunchConfig_t cfg = {};
@@ -777,13 +779,15 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     // as a programmatic dependent of the first part
     vd::EvictArgs a1 = a;
     a1.cluster = 1;
+    a1.let_next = 1;
     const size_t smem1 = vd::smem_layout(c->capacity, 1, kind).total;
     if (smem1 > (size_t)st->smem_optin) return VD_ERR_UNSUPPORTED;
-    r = launch(kern, solo, 1, smem1, &a1, s);
+    r = launch(kern, solo, 1, smem1, &a1, s, true);
     if (r != VD_OK) return r;
     // the second part's per-unit pointers start at unit `solo`
     const size_t rows = (size_t)solo * c->capacity, dd = (size_t)c->head_dim;
     a.unit_base = (int32_t)solo;
+    a.wait_first = 0;  // it runs beside the first part
     a.k += rows * dd;
     a.v += rows * dd;
     if (a.running_sum) a.running_sum += (size_t)solo * dd;
@@ -797,7 +801,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     if (a.v_new) a.v_new += (size_t)solo * a.B * dd;
     r = launch(kern, units - solo, a.cluster, smem, &a, s, true);
   } else {
-    r = launch(kern, units, a.cluster, smem, &a, s);
+    r = launch(kern, units, a.cluster, smem, &a, s, true);
   }
   return r != VD_OK || score_only ? r : clamp_lengths();
 }

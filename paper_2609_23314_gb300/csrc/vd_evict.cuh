@@ -184,6 +184,8 @@ struct EvictArgs {
   // launch's first one.  Only the sequence index adds it; every per-unit
   // pointer above comes offset to the launch's first unit.
   int32_t unit_base;
+  int32_t wait_first;  // 1: wait for the previous kernel on the stream before reading
+  int32_t let_next;    // 1: let the next kernel on the stream be scheduled at once
 };
 
 // Fixed part of the dynamic shared memory.  After it (16-byte aligned): the
@@ -1992,14 +1994,18 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
   if (DECODE && C > 1) cluster_wait();
 }
 
-// One unit per cluster of C CTAs (evict_unit).  Split launches (the host's
-// split_plan) run the units in two launches on one stream, the second a
-// programmatic dependent launch whose CTAs take the slots the first leaves
-// free.  So every kernel lets its dependents be scheduled at once.  The two
-// parts touch disjoint units, so the second reads nothing the first writes;
-// it waits for the first only before it ends (griddepcontrol.wait, a no-op
-// in a normal launch), so that work queued after it on the stream also
-// follows the first.
+// One unit per cluster of C CTAs (evict_unit).  Launched as a programmatic
+// dependent of the previous kernel on the stream, which it waits for first
+// (wait_first).  Split launches (the host's split_plan) run the units in two
+// launches on one stream, the second a programmatic dependent whose CTAs take
+// the slots the first leaves free: so the first, and every eviction (for its
+// length update), lets its dependents be scheduled at once (let_next).  A
+// score-only launch that could be followed by another does not: the next
+// one's CTAs would fill the slots that happen to be free, and unevenly
+// (prefill_wide's scores 204 -> 226 us).  The two parts touch disjoint units, so the second reads
+// nothing the first writes (what both read is older than the first, whose
+// CTAs have all waited by then); it waits for the first only before it ends, so
+// that work queued after it on the stream also follows the first.
 template <int VAR, bool DECODE, bool HF, bool FUSED, bool GEN, bool SCORE = false>
 __global__ void __launch_bounds__(kThreads, SCORE    ? VD_SCORE_MIN_CTAS
                                             : GEN    ? VD_GENERAL_MIN_CTAS
@@ -2007,7 +2013,8 @@ __global__ void __launch_bounds__(kThreads, SCORE    ? VD_SCORE_MIN_CTAS
                                             : HF     ? VD_HF_BLOCK_MIN_CTAS
                                                      : VD_BLOCK_MIN_CTAS)
     evict_kernel(const EvictArgs a) {
-  grid_launch_dependents();
+  if (a.wait_first) grid_dependency_wait();
+  if (a.let_next) grid_launch_dependents();
   evict_unit<VAR, DECODE, HF, FUSED, SCORE, GEN>(a);
   grid_dependency_wait();
 }
