@@ -40,12 +40,16 @@ static __device__ unsigned g_vd_status;
 
 // ---------------------------------------------------------------------------
 // small kernels: append (Eq. block_processing's concatenation), length
-// update after an eviction, and the from-scratch running sum
+// update after an eviction, and the from-scratch running sum.  The append and
+// the length updates are programmatic dependents of the kernel before them
+// (launch_dependent) and wait for it before they read anything.
 // ---------------------------------------------------------------------------
 __global__ void vd_append_kernel(uint16_t* __restrict__ k, uint16_t* __restrict__ v,
                                  const uint16_t* __restrict__ kn, const uint16_t* __restrict__ vn,
                                  const int32_t* __restrict__ len, int units_per_seq,
                                  long long n_units, int cap, int d, int B, unsigned* status) {
+  vd::grid_dependency_wait();
+  vd::grid_launch_dependents();
   const int d8 = d >> 3;
   const long long total = n_units * (long long)B * d8;
   for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < total;
@@ -67,6 +71,7 @@ __global__ void vd_append_kernel(uint16_t* __restrict__ k, uint16_t* __restrict_
 }
 
 __global__ void vd_len_add_kernel(int32_t* len, int n_seq, int cap, int B) {
+  vd::grid_dependency_wait();
   const int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n_seq) return;
   const int n = len[s];
@@ -545,6 +550,27 @@ bool cached_fits(const void* kern, long long groups, int c, size_t smem, DeviceS
   return fits;
 }
 
+// A plain kernel of kThreads-thread blocks as a programmatic dependent launch
+// (it waits in griddepcontrol.wait before its first access to memory).
+template <class... Params, class... Args>
+vd_status launch_dependent(unsigned blocks, cudaStream_t s, void (*kern)(Params...),
+                           Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(blocks);
+  cfg.blockDim = dim3(kThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(args)...) != cudaSuccess) {
+    cudaGetLastError();
+    return VD_ERR_CUDA;
+  }
+  return VD_OK;
+}
+
 vd_status launch(const void* kern, long long groups, int c, size_t smem, const void* params,
                  cudaStream_t s, bool dependent = false) {
   cudaLaunchConfig_t cfg = {};
@@ -722,24 +748,11 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   a.unit_base = 0;
   a.wait_first = 1;
   a.let_next = score_only ? 0 : 1;
-  // the eviction's length update, a programmatic dependent of it
-  auto clamp_lengths = [&]() -> vd_status {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)((c->n_seq + kThreads - 1) / kThreads));
-    cfg.blockDim = dim3(kThreads);
-    cfg.stream = s;
-    cudaLaunchAttribute pdl;
-    pdl.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    pdl.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &pdl;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, vd_len_clamp_kernel, c->len, N_dev, N, c->n_seq, c->capacity,
-                           (int)a.B, (int)a.mu_running, decode ? 1 : 0, fused ? (int)a.B : 0) !=
-        cudaSuccess) {
-      cudaGetLastError();
-      return VD_ERR_CUDA;
-    }
-    return VD_OK;
+  // the eviction's length update
+  auto clamp_lengths = [&]() {
+    return launch_dependent((unsigned)((c->n_seq + kThreads - 1) / kThreads), s,
+                            vd_len_clamp_kernel, c->len, N_dev, N, c->n_seq, c->capacity, (int)a.B,
+                            (int)a.mu_running, decode ? 1 : 0, fused ? (int)a.B : 0);
   };
   if (use_small(c, score_only, holefill, disp_out, *st)) {
     const void* sk = small_kernel(var, decode, fused);
@@ -916,13 +929,13 @@ vd_status vd_append(const vd_cache* c, const void* k_new, const void* v_new, int
   const long long work = units * B * (c->head_dim / 8);
   const long long want = (work + 255) / 256;
   const int blocks = (int)(want < (long long)st->sms * 32 ? want : (long long)st->sms * 32);
-  vd_append_kernel<<<blocks, 256, 0, s>>>(
-      static_cast<uint16_t*>(c->k), static_cast<uint16_t*>(c->v),
-      static_cast<const uint16_t*>(k_new), static_cast<const uint16_t*>(v_new), c->len,
-      c->n_layer * c->n_kv_head, units, c->capacity, c->head_dim, B, st->status);
-  vd_len_add_kernel<<<(c->n_seq + 255) / 256, 256, 0, s>>>(c->len, c->n_seq, c->capacity, B);
-  if (cudaGetLastError() != cudaSuccess) return VD_ERR_CUDA;
-  return VD_OK;
+  r = launch_dependent((unsigned)blocks, s, vd_append_kernel, static_cast<uint16_t*>(c->k),
+                       static_cast<uint16_t*>(c->v), static_cast<const uint16_t*>(k_new),
+                       static_cast<const uint16_t*>(v_new), c->len, c->n_layer * c->n_kv_head,
+                       units, c->capacity, c->head_dim, B, st->status);
+  if (r != VD_OK) return r;
+  return launch_dependent((unsigned)((c->n_seq + kThreads - 1) / kThreads), s, vd_len_add_kernel,
+                          c->len, c->n_seq, c->capacity, B);
 }
 
 vd_status vd_running_sum_init(const vd_cache* c, double* running_sum, vd_stream_t stream) {

@@ -476,6 +476,7 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
     for (int i = 0; i <= kResChunks; ++i) mbar_init(bar_s + 8u * (uint32_t)i, 1);
     fence_mbar_init();
   }
+  __syncthreads();
   grid_dependency_wait();
   const int C = a.cluster, d = a.d, d8 = d >> 3, lpr = a.lpr, cap = a.capacity;
   const ResLayout L = resident_layout(cap, d, C, DECODE, HF, a.mu_running != 0, ra.both != 0);
@@ -489,7 +490,8 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
   const unsigned rank = C > 1 ? cluster_ctarank() : 0u;
   const int u = C > 1 ? (int)cluster_id_x() : (int)blockIdx.x;
   const int seq = u / a.units_per_seq;
-  const int len0 = a.len[seq];
+  // from L2: the previous launch may have set it while this one was resident
+  const int len0 = __ldcg(a.len + seq);
   const int n = len0 + (FUSED ? a.B : 0);
   const int Nb = a.N_dev ? a.N_dev[seq] : a.N;
   uint16_t* kb = a.k + (size_t)u * cap * d;
@@ -576,7 +578,6 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
     else if (!HF && !DECODE && fs > 0)  // on its way to L2 while the scores and the select run
       bulk_prefetch_l2(ob + (size_t)r0 * d, (uint32_t)(fs * row_bytes));
   }
-  __syncthreads();
   auto ld_row = [&](int j, int ci) {
     return *reinterpret_cast<const uint4*>(smem_raw + L.buf + (size_t)(j * row_bytes + ci * 16));
   };

@@ -140,7 +140,8 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
   // writes nothing but still reaches the cluster barrier
   const bool unit_ok = u < sa.n_units;
   const int seq = unit_ok ? u / a.units_per_seq : 0;
-  const int len0 = unit_ok ? a.len[seq] : -1;
+  // from L2: the previous launch may have set it while this one was resident
+  const int len0 = unit_ok ? __ldcg(a.len + seq) : -1;
   const int n = len0 + (FUSED ? a.B : 0);
   const int Nb = unit_ok ? (a.N_dev ? a.N_dev[seq] : a.N) : 0;
   const size_t ubase = (size_t)u * cap * d;
