@@ -303,9 +303,9 @@ bool cluster_allowed(int c, int d) {
 // SM only share its bandwidth while every cluster barrier still costs.
 // `side` is the largest C with units * C <= 2.6 SMs that leaves a CTA at least
 // kMinRowsPerCta rows.  It is taken by ordered block eviction unless its
-// slices exceed 1.25 MB (300 KB where the mean is recomputed, `resum`: 288
-// units of 2176 rows C = 2 146 us, C = 1 156), by hole-fill decode and by score-only launches without
-// the bulk ring.  d = 128, us: ordered block, n = 1152, 96 units C = 4 39.0
+// slices exceed 1.25 MB (where the mean is recomputed, `resum`, the lines of the
+// next paragraph), by hole-fill decode and by score-only launches without the
+// bulk ring.  d = 128, us: ordered block, n = 1152, 96 units C = 4 39.0
 // (C = 2 42, 8 58), 192 units C = 2 55 (1 61, 4 73), 240 units C = 1 66.6
 // (2 69.5, 8 115); n = 2176, 288 units C = 1 131 (2 136); where the score pass
 // is bound by instruction issue (`heavy`: Dir, or a head dim off the batched
@@ -319,7 +319,16 @@ bool cluster_allowed(int c, int d) {
 // whose tail shrinks with the slice.  The smallest C with slices of at most
 // 300 KB: 164 KB units C = 1 (800 units 102 us; C = 2 111, 4 158), 557 KB
 // units C = 2 (800 units 344; C = 1 361), prefill_wide's 2.2 MB C = 8 (568 us;
-// C = 4 586, C = 1 612).  Ordered decode, which has no select to synchronise
+// C = 4 586, C = 1 612).  With a recomputed mean C = 2 only up to 185 KB (288
+// units of 2176 rows C = 4 146.4 us, C = 2 149, C = 1 154; 800 units of 1828
+// rows C = 4 309, C = 2 321; d = 64, 2828 rows, 181 KB, C = 2 253, C = 4 264);
+// it is bound by more instructions per row, so a short last wave costs more.
+// Where that C makes 1 to 1.5 waves, the largest C within one wave is taken (192
+// units of 2176 rows, recomputed, C = 2 107, C = 4 109; Dir, 288 units, C = 1 179,
+// C = 2 198), for a batched score pass with a recomputed mean only if its slices
+// stay within 300 KB (160 units of 4224 rows C = 4 176, C = 2 198); if not even
+// C = 1 is within one wave, the next C (Dir, 480 units of 1152 rows C = 2 142, C
+// = 1 152; 640 units, L2, C = 2 151, C = 1 161).  Ordered decode, which has no select to synchronise
 // on: the largest C within 0.85 of a wave, or the smallest (up to 4) with
 // slices of at most 200 KB where that is larger (n = 4097, 128 units C = 4
 // 79.7 us, C = 2 86; 16384 units C = 4 7.28 ms, C = 1 7.37; n = 3001, 800
@@ -347,6 +356,12 @@ int choose_cluster(const void* kern, long long units, int d, int capacity, int k
                    size_t* smem_out) {
   int roomy = 0, smallest = 0, narrow = 0;  // see above
   int side = 0, sliced = 0, filled = 0, waved = 0;
+  int single = 0, next = 0;      // largest C in one wave; first C above `sliced`
+  double sliced_waves = 0;
+  auto slice_of = [&](int c) { return (long long)((capacity + c - 1) / c) * d * 2; };
+  auto most_of = [&](int c) {  // the largest slice for C = c, see above
+    return kind == vd::kKindDecode ? 200LL << 10 : resum && !heavy && c == 2 ? 185LL << 10 : 300LL << 10;
+  };
   for (int c = 1; c <= 16; c *= 2) {
     if (want >= 1 && c != want) continue;
     if ((d / 8 * 2) % c) continue;
@@ -372,7 +387,12 @@ int choose_cluster(const void* kern, long long units, int d, int capacity, int k
     if (room) roomy = c;
     if (room && (heavy ? waves <= 0.95 : (double)(units * c) <= 2.6 * st.sms)) side = c;
     if (room && waves <= 0.85) filled = c;
-    if (sliced == 0 && rows * d * 2 <= (kind == vd::kKindDecode ? 200 << 10 : 300 << 10)) sliced = c;
+    if (waves <= 1.0) single = c;
+    if (sliced != 0 && next == 0 && room) next = c;
+    if (sliced == 0 && slice_of(c) <= most_of(c)) {
+      sliced = c;
+      sliced_waves = waves;
+    }
     const bool enough = kind == vd::kKindBlock       ? waves >= 0.4
                         : kind == vd::kKindScoreBulk ? waves >= 0.5
                                                      : waves <= 1.0 || waves >= 2.0;
@@ -385,9 +405,11 @@ int choose_cluster(const void* kern, long long units, int d, int capacity, int k
   } else if (kind == vd::kKindScoreBulk || (kind == vd::kKindBlock && holefill)) {
     chosen = waved ? waved : large;
   } else if (kind == vd::kKindBlock) {
-    const bool fits_side =
-        side && (long long)((capacity + side - 1) / side) * d * 2 <=
-                    (resum ? 300 << 10 : (5LL << 20) / 4);
+    const bool fits_side = side && slice_of(side) <= (resum ? most_of(side) : (5LL << 20) / 4);
+    if (sliced_waves > 1.0 && sliced_waves < 1.5) {
+      if (single && (!resum || heavy || slice_of(single) <= 300 << 10)) sliced = single;
+      else if (!single && next) sliced = next;
+    }
     chosen = fits_side ? side : sliced ? sliced : large;
   } else if (kind == vd::kKindDecode && !holefill) {
     chosen = std::max(filled, std::min(sliced ? sliced : large, 4));
@@ -603,9 +625,9 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
 // rows, d = 128: 167 us against 136).  C is the largest size, up to 12, that
 // leaves a CTA at least 64 rows and the launch at most two CTAs per SM (decode,
 // which has fewer phases: three), and whose clusters form one wave.  Measured, streaming / resident, d = 128,
-// n = 2176: 8 units 29.0 / 19.6 us (C = 12; C = 8 20.9), 16 units 31.5 / 22.1
-// (C = 10), 32 units 35.1 / 29.3 (C = 8; C = 4 30.6); n = 1152: 96 units
-// 57.2 / 33.3 (C = 3; C = 4, 2.5 CTAs per SM, 50.3).  Both tensors get a
+// n = 2176: 8 units 24.9 / 18.2 us (C = 12; C = 8 1.3 us more), 16 units 27.3 /
+// 21.5 (C = 10), 32 units 30.6 / 29.0 (C = 8; C = 4 1.3 us more); n = 1152: 96
+// units 34.4 / 33.7 (C = 3; C = 4, 2.5 CTAs per SM, 50.3).  Both tensors get a
 // buffer where that keeps the wave (8 units 17.6 us in the kernel against
 // 20.3).  More units, or larger ones: C = 1 where three CTAs share an SM (decode:
 // two), in any number of waves, since a small unit is only its phases in either
@@ -613,9 +635,9 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
 // units 208 / 182; d = 96, 240 rows, 1600 units 105 / 86 (340 rows, two CTAs per
 // SM, 110 / 127); decode, d = 128, 301 rows, 640 units 42.9 / 33.7, 4800 units
 // 197 / 172 (451 rows, one CTA per SM, 249 / 328).  A hole-fill block event moves
-// so few rows that the streaming kernel catches up at 18 MB of scored rows (d =
-// 256, 1128 rows, 16 units 25.3 / 22.6, 32 units 27.6 / 29.7); otherwise the same
-// lines: hole-fill block, d = 128, 2176 rows, 8 units 22.8 / 18.0, 230 rows, 320
+// so few rows that the streaming kernel catches up at 12 MB of scored rows (d =
+// 256, 1128 rows, 16 units 23.4 / 23.1, 24 units 24.6 / 27.5); otherwise the same
+// lines: hole-fill block, d = 128, 2176 rows, 8 units 20.6 / 17.9, 230 rows, 320
 // units 39.1 / 20.1; hole-fill decode, 4097 rows, 8 units 19.2 / 11.0, 201 rows,
 // 4800 units 138 / 86.  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
 // c CTAs (100 + c: with both buffers), for tests.  Returns C, or 0.
@@ -662,7 +684,7 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
         if (at_once(c, false) >= units) break;
       both = !holefill && c >= 1 && at_once(c, true) >= units;
     }
-    if (holefill && !decode && c > 1 && units * capacity * d * 2 > 18LL << 20) c = 0;
+    if (holefill && !decode && c > 1 && units * capacity * d * 2 > 12LL << 20) c = 0;
     if (c < 1 && at_once(1, false) >= (decode ? 2LL : 3LL) * st.sms) c = 1;
   }
   const size_t smem = c >= 1 ? smem_of(c, both) : 0;
