@@ -926,7 +926,7 @@ def measure_dispersion(args, device, variant, peak, rank):
 
     ms_re = timed(vd.VD_MU_RECOMPUTE)
     ms = timed(vd.VD_MU_RUNNING)
-    kernel = "vd::evict_kernel<0, true, false, false, true> (score only)"
+    kernel = "vd::evict_kernel<0, true, false, false, false, true> (score only)"
     # the realized sigma_V / sigma_K of the generator (untimed)
     sigma_k = torch.empty_like(sigma)
     vd.vd_score_ex(w.cache, vd.VD_SCORE_L2, True, None, sigma_k)
@@ -1118,7 +1118,8 @@ def run_vd(args):
         achieved = alg / (kern_ms / 1e3) / 1e9
         kernel = (f"vd::evict_kernel<{variant}, {str(isinstance(w, Decode)).lower()}, "
                   f"{str(layout == 'holefill').lower()}, "
-                  f"{str(getattr(w, 'fused', False)).lower()}>")
+                  f"{str(getattr(w, 'fused', False)).lower()}, "
+                  f"{str(variant == vd.VD_SCORE_DIR or w.d not in (64, 128, 256)).lower()}>")
         mu_name = "running" if mm == vd.VD_MU_RUNNING else "recompute"
         traffic = None
         if not (set(opts) - {"separate_append"}):   # scoring options: never captured

@@ -21,7 +21,9 @@
 //             For d = 64, 128, 256 (L2, Norm) each lane keeps
 //             a batch of 8 rows' partial sums (packed f32x2 arithmetic) and
 //             the batch is reduced with a transposed butterfly
-//             (score_rows_fast).  Scores become order-preserving uint32 keys.
+//             (score_rows_fast); other head dims and Dir take smaller batches
+//             of row pairs (score_rows_general).  Scores become
+//             order-preserving uint32 keys.
 //   3. select block prompt processing (N+B -> N): a 4-pass 8-bit radix select
 //             for the N-th largest key t; every CTA histograms only its own
 //             rows and the cluster adds the C histograms through DSMEM.
@@ -46,7 +48,8 @@
 //
 // Template flags select the rest at compile time: DECODE (the arg-min path),
 // HF (hole-fill layout: ties broken by token position, and only the kept rows
-// at or above N move, into the evicted slots below N) and FUSED (the rows at
+// at or above N move, into the evicted slots below N), GEN (score_rows_general,
+// with the registers of 3 CTAs per SM) and FUSED (the rows at
 // or above len are read from the caller's staging buffers and written only
 // if they survive: the append of Eq. block_processing fused into the event).
 //

@@ -25,7 +25,7 @@
 // Bound by the latency of these steps.  The rows arrive by bulk copies (K while
 // V is scored), the running sum is read before they land, rows are scored four
 // at a time and compacted two at a time: 2 units of 160 rows, d = 64, 9.2 ->
-// 8.1 us a call.  Up to 256 rows: beyond, the comparisons cost more than the
+// 7.8 us a call.  Up to 256 rows: beyond, the comparisons cost more than the
 // resident kernel's histogram and second launch (d = 64, 256 rows 9.9 us against
 // 11.8; d = 32, 384 rows 14.4 against 12.0; d = 16, 1000 rows 45.7 against 13.0).
 // With many units three CTAs share an SM; us, streaming kernel / this one: d =

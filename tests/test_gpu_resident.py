@@ -1,7 +1,7 @@
 """The resident kernel (a unit's scored rows in the shared memory of its
 cluster) against the streaming kernel on the same inputs, over the forms it
-accepts: rules, mean modes, fused and two-call, block and decode, scoring
-options, ragged lengths and budgets, cluster sizes that divide nothing, slices
+accepts: both layouts, rules, mean modes, fused and two-call, block and decode,
+scoring options, ragged lengths and budgets, cluster sizes that divide nothing, slices
 that end mid-row-group or are empty, heavy ties and non-finite rows.
 VD_RESIDENT=0 forces the streaming kernel, VD_RESIDENT=c the resident one on
 clusters of c CTAs (100 + c: both tensors resident).  Needs a GB300.
