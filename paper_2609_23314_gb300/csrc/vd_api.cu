@@ -46,7 +46,7 @@ static __device__ unsigned g_vd_status;
 // ---------------------------------------------------------------------------
 __global__ void vd_append_kernel(uint16_t* __restrict__ k, uint16_t* __restrict__ v,
                                  const uint16_t* __restrict__ kn, const uint16_t* __restrict__ vn,
-                                 const int32_t* __restrict__ len, int units_per_seq,
+                                 const int32_t* len, int units_per_seq,
                                  long long n_units, int cap, int d, int B, unsigned* status) {
   vd::grid_dependency_wait();
   vd::grid_launch_dependents();
@@ -58,7 +58,8 @@ __global__ void vd_append_kernel(uint16_t* __restrict__ k, uint16_t* __restrict_
     const long long ub = idx / d8;
     const int b = (int)(ub % B);
     const long long u = ub / B;
-    const int n = len[u / units_per_seq];
+    // from L2: the previous kernel may set it while this one is resident
+    const int n = __ldcg(len + u / units_per_seq);
     if (n < 0 || n > cap - B) {
       if (b == 0 && c == 0 && u % units_per_seq == 0) vd::record_status(status, vd::kStDeviceLen);
       continue;
