@@ -32,7 +32,7 @@
  *   budget) never trap: the kernel records the first one in the device status
  *   word (read it with vd_get_device_status) and leaves the affected unit
  *   untouched, except VD_ERR_NONFINITE, which is recorded while the unit is
- *   still evicted with NaN scores ranked lowest.
+ *   still evicted with NaN scores ranked lowest, and VD_ERR_TIMEOUT (below).
  * - Precision: scores are computed in fp32 from bf16 inputs against the
  *   cache mean carried as an fp32 part plus its fp32 remainder; the mean is
  *   accumulated with exact (TwoSum) fp32 sums, or from the fp64 running sum,
@@ -77,8 +77,17 @@ typedef enum {
                              C <= head_dim / 4): at head_dim >= 64 every
                              capacity up to 65536 fits */
   VD_ERR_NONFINITE = 4,   /* device: a score was NaN or infinite */
-  VD_ERR_TIMEOUT = 5,     /* device: a bounded wait for a bulk copy gave up (score-only
-                             kernels); that call's outputs are unspecified */
+  VD_ERR_TIMEOUT = 5,     /* device: a bounded wait for a bulk copy gave up (never
+                             expected).  Score-only calls: the outputs are
+                             unspecified.  Evictions: the call's scores and sigma
+                             are unspecified, and the lengths of the sequences it
+                             happened in stay as they were before the eviction.
+                             Of such a sequence, units whose copies landed may
+                             have been evicted all the same; the others' K, V,
+                             positions and running sums are untouched, except
+                             where the second tensor's copy gave up after the
+                             first one had been compacted: that unit's contents
+                             are unspecified.  Fill the sequence again */
   VD_ERR_CUDA = 6,        /* a CUDA runtime call failed (launch error, ...) */
   VD_ERR_DEVICE_LEN = 7,  /* device: len[s] out of [0, capacity], or len + B > capacity
                              on append, or B > len in running-sum mode */

@@ -92,6 +92,10 @@ __global__ void vd_len_clamp_kernel(int32_t* len, const int32_t* N_dev, int N, i
   const int n0 = len[s];
   const int n = n0 + added;
   const int Nb = N_dev ? N_dev[s] : N;
+  if (vd::len_marked(n0)) {  // a unit was not evicted: the length stays
+    len[s] = vd::mark_len(0) - n0;
+    return;
+  }
   if (n0 < 0 || n > cap || (running && B > n)) return;
   if (Nb < 1 || Nb > N) return;
   if (n <= Nb) {
@@ -649,7 +653,7 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
                   bool holefill, bool running, DeviceState& st, size_t* smem_out, bool* both_out) {
   const char* env = std::getenv("VD_RESIDENT");
   const int want = env ? std::atoi(env) : -1;
-  if (want == 0 || std::getenv("VD_CLUSTER_SIZE") || capacity > 32768) return 0;
+  if (want == 0 || std::getenv("VD_CLUSTER_SIZE") || capacity > vd::kMaxMarkedLen) return 0;
   const int kind = kResidentKind + (running ? 1 : 0);
   {
     std::lock_guard<std::mutex> lk(g_mu);
@@ -697,6 +701,18 @@ int resident_plan(const void* kern, long long units, int d, int capacity, bool d
   *smem_out = smem;
   *both_out = both;
   return c;
+}
+
+// Polls after which a device wait gives up.  VD_WAIT_LIMIT=a or a:b lowers them,
+// for tests (a for the scored rows' copies, b for the other tensor's; 0: at once).
+void wait_limits(uint32_t* scored, uint32_t* other) {
+  *scored = *other = vd::kWaitLimit;
+  const char* s = std::getenv("VD_WAIT_LIMIT");
+  if (!s) return;
+  char* end = nullptr;
+  *scored = (uint32_t)std::min<unsigned long>(std::strtoul(s, &end, 10), vd::kWaitLimit);
+  if (*end == ':')
+    *other = (uint32_t)std::min<unsigned long>(std::strtoul(end + 1, nullptr, 10), vd::kWaitLimit);
 }
 
 vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_variant var,
@@ -771,6 +787,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   a.unit_base = 0;
   a.wait_first = 1;
   a.let_next = score_only ? 0 : 1;
+  wait_limits(&a.wait_limit, &a.wait_limit_other);
   // the eviction's length update
   auto clamp_lengths = [&]() {
     return launch_dependent((unsigned)((c->n_seq + kThreads - 1) / kThreads), s,

@@ -26,6 +26,16 @@ __device__ __forceinline__ void record_status(unsigned* st, unsigned code) {
   atomicCAS(st, 0u, code);
 }
 
+// A sequence with a unit whose copies did not land in time keeps its length.
+// The unit leaves it marked for the length update that follows on the stream,
+// which puts it back; the sequence's units that read it only then see a length
+// out of range and leave themselves alone too.
+constexpr int kMaxMarkedLen = 32768;  // the largest capacity of the kernels that mark
+__host__ __device__ constexpr int mark_len(int len) { return -(1 << 30) - len; }
+__host__ __device__ constexpr bool len_marked(int len) {
+  return len <= mark_len(0) && len >= mark_len(kMaxMarkedLen);
+}
+
 // ---------------------------------------------------------------------------
 // bf16 <-> fp32.  A bf16 value is the upper half of an fp32 bit pattern, so
 // widening is a shift; eight values arrive per 16-byte vector.
@@ -220,10 +230,13 @@ __device__ __forceinline__ void bulk_g2s(uint32_t dst, const void* src, uint32_t
 
 // Waits until the barrier's phase with the given parity has completed, for
 // at most `limit` polls.  Returns false (and records kStTimeout) if it gave
-// up: the caller then goes on with whatever the buffer holds, so that the
-// kernel still ends and every barrier of the CTA or cluster is still reached.
+// up.  The kernel still ends and every barrier of the CTA or cluster is still
+// reached: the caller may compute on whatever the buffer holds, but stores
+// nothing made from it in the cache, and before it leaves, or uses the buffer
+// again, thread 0 waits for the copy once more, with the full limit.
+constexpr unsigned kWaitLimit = 1u << 22;
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned* status,
-                                          unsigned limit = 1u << 22) {
+                                          unsigned limit) {
   for (unsigned i = 0; i < limit; ++i) {
     uint32_t done;
     asm volatile(

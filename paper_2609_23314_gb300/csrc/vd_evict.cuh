@@ -189,6 +189,9 @@ struct EvictArgs {
   int32_t unit_base;
   int32_t wait_first;  // 1: wait for the previous kernel on the stream before reading
   int32_t let_next;    // 1: let the next kernel on the stream be scheduled at once
+  // polls of an mbarrier after which a wait gives up: for the scored rows, and
+  // for the other tensor's (kWaitLimit, fewer only in tests)
+  uint32_t wait_limit, wait_limit_other;
 };
 
 // Fixed part of the dynamic shared memory.  After it (16-byte aligned): the
@@ -719,23 +722,25 @@ static_assert(kBulkStages >= 2 && kBulkStages <= 4, "bulk ring: 2 to 4 stages (S
 struct BulkRing {
   uint32_t ring, bar0;
   int gst;
+  unsigned limit;  // polls after which a wait gives up
 };
 
-__device__ __forceinline__ BulkRing bulk_ring_init(uint32_t ring, Smem& S) {
+__device__ __forceinline__ BulkRing bulk_ring_init(uint32_t ring, Smem& S, unsigned limit) {
   const uint32_t bar0 = smem_addr(&S.bar[0]);
   if (threadIdx.x == 0) {
     for (int sl = 0; sl < kBulkStages; ++sl) mbar_init(bar0 + 8u * (uint32_t)sl, 1);
     fence_mbar_init();
   }
   __syncthreads();
-  return {ring, bar0, 0};
+  return {ring, bar0, 0, limit};
 }
 
 // Streams nst stages of the rows at `base` (row_bytes each); stage_rows(i,
 // first, count) names stage i's rows [first, first + count).  Thread 0 issues
 // each stage as one bulk copy; every thread waits for it, consume(first,
 // count, stage address) reads it, and a block barrier frees the slot before
-// thread 0 refills it.
+// thread 0 refills it.  A thread whose wait gives up consumes what the slot holds:
+// the call's outputs are unspecified then.
 template <class StageRows, class Consume>
 __device__ __forceinline__ void bulk_stream(BulkRing& br, const uint16_t* base, int nst,
                                             int row_bytes, StageRows stage_rows, Consume consume,
@@ -756,7 +761,9 @@ __device__ __forceinline__ void bulk_stream(BulkRing& br, const uint16_t* base, 
   for (int i = 0; i < nst; ++i) {
     const int g = br.gst + i;
     const uint32_t sl = (uint32_t)(g % kBulkStages);
-    mbar_wait(br.bar0 + 8u * sl, (uint32_t)(g / kBulkStages) & 1u, status);
+    const uint32_t bar = br.bar0 + 8u * sl, parity = (uint32_t)(g / kBulkStages) & 1u;
+    if (!mbar_wait(bar, parity, status, br.limit) && threadIdx.x == 0)
+      mbar_wait(bar, parity, status, kWaitLimit);  // before the slot is refilled
     int first, count;
     stage_rows(i, first, count);
     consume(first, count, br.ring + sl * (uint32_t)kBulkStageBytes);
@@ -1571,8 +1578,8 @@ __device__ __forceinline__ void evict_unit(const EvictArgs& a) {
     return;
   }
   if (score_only && n == 0) return;
-  BulkRing br{0u, 0u, 0};
-  if constexpr (bulk) br = bulk_ring_init(ring, S);
+  BulkRing br{0u, 0u, 0, 0u};
+  if constexpr (bulk) br = bulk_ring_init(ring, S, a.wait_limit);
 
   // column slice of [K | V] this CTA compacts; the running sum is kept for
   // the part of it that lies in the scored tensor (V, or K for the key-side

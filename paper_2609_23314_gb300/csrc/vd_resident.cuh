@@ -65,11 +65,13 @@ struct ResSmem {
   // are dead between the scores and the retired rows' sum
   double snew[256];  // running mode: the running sum plus the appended rows
   unsigned long long bar[kResChunks + 1];  // scored tensor's chunks, other tensor
-  unsigned long long best[kResMaxCluster];  // decode: every CTA's minimum (pushed by it)
+  // decode: every CTA's minimum (pushed by it); the last entry: kLostBest where a
+  // wait in the cluster gave up
+  unsigned long long best[kResMaxCluster + 1];
   int best_slot[kResMaxCluster];            // hole-fill decode: its slot (pushed)
   int wslot[kWarps];
   uint32_t kmin[kResMaxCluster];  // every CTA's smallest and largest key (pushed)
-  uint32_t kmax[kResMaxCluster];
+  uint32_t kmax[kResMaxCluster + 1];  // (the last entry: kLostKey, as for best)
   unsigned long long wbest[kWarps];
   uint32_t wmin[kWarps], wmax[kWarps];
   int scan[kWarps], pre[kWarps];
@@ -81,7 +83,12 @@ struct ResSmem {
   float fsh[kWarps];
   float inv_mnorm;
   int mu_zero;
+  int lost;  // a wait for this CTA's scored rows gave up
 };
+// Values that no minimum and no key has: they win the exchange's min and max, so
+// that the outcome needs no load of its own.
+constexpr unsigned long long kLostBest = 0ull;
+constexpr uint32_t kLostKey = 0xffffffffu;
 static_assert(kResBuckets * 4 == 4 * 256 * 4, "the histogram covers mu .. acc_lo");
 
 __host__ __device__ inline int resident_rows(int n, int c) {
@@ -475,6 +482,9 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
   if (threadIdx.x == 0) {
     for (int i = 0; i <= kResChunks; ++i) mbar_init(bar_s + 8u * (uint32_t)i, 1);
     fence_mbar_init();
+    S.lost = 0;
+    S.best[kResMaxCluster] = ~0ull;
+    S.kmax[kResMaxCluster] = 0u;
   }
   __syncthreads();
   grid_dependency_wait();
@@ -578,6 +588,28 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
     else if (!HF && !DECODE && fs > 0)  // on its way to L2 while the scores and the select run
       bulk_prefetch_l2(ob + (size_t)r0 * d, (uint32_t)(fs * row_bytes));
   }
+  // A wait that gives up goes on with whatever the buffer holds (shared memory
+  // only, every index clamped) up to the exchange of step 4, before the first
+  // store to the cache.  There the cluster agrees, waits for its copies in flight
+  // and leaves the unit as it is.
+  auto tell_lost = [&](unsigned cc) {  // to CTA cc of the cluster
+    if (DECODE) {
+      if (C > 1) st_cluster_u64(mapa(smem_addr(&S.best[kResMaxCluster]), cc), kLostBest);
+      else S.best[kResMaxCluster] = kLostBest;
+    } else {
+      if (C > 1) st_cluster_u32(mapa(smem_addr(&S.kmax[kResMaxCluster]), cc), kLostKey);
+      else S.kmax[kResMaxCluster] = kLostKey;
+    }
+  };
+  auto leave_unit = [&]() {
+    if (tid != 0) return;
+    for (int i = 0; i < nch; ++i) mbar_wait(bar_s + 8u * (uint32_t)i, 0u, a.status, kWaitLimit);
+    if (!HF && ra.both) mbar_wait(bar_o, 0u, a.status, kWaitLimit);
+    if (rank == 0) {
+      __threadfence();  // the status first
+      a.len[seq] = mark_len(len0);
+    }
+  };
   auto ld_row = [&](int j, int ci) {
     return *reinterpret_cast<const uint4*>(smem_raw + L.buf + (size_t)(j * row_bytes + ci * 16));
   };
@@ -611,7 +643,8 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
               },
               [](int) { return 1.f; }, scratch);
       } else {
-        for (int i = 0; i < nch; ++i) mbar_wait(bar_s + 8u * (uint32_t)i, 0u, a.status);
+        for (int i = 0; i < nch; ++i)
+          if (!mbar_wait(bar_s + 8u * (uint32_t)i, 0u, a.status, a.wait_limit)) S.lost = 1;
         t = resident_sum<4>(d, lpr, R, ld_row, [](int) { return 1.f; }, scratch);
       }
       if (C > 1 && !alone) {
@@ -696,7 +729,7 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
       }
     };
     for (int i = 0; i < nch; ++i) {
-      mbar_wait(bar_s + 8u * (uint32_t)i, 0u, a.status);
+      if (!mbar_wait(bar_s + 8u * (uint32_t)i, 0u, a.status, a.wait_limit)) S.lost = 1;
       const int x = i * rch, y = min(R, x + rch);
       if (VAR != 1 && d == 128)
         resident_score_fast<VAR, 16>(sbuf, x, y, S.mu, S.mulo, finish);
@@ -749,11 +782,14 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
         S.best[0] = b;
         S.best_slot[0] = bs;
       }
+      if (S.lost) tell_lost((unsigned)tid);
     }
-    if (!HF && ra.both) mbar_wait(bar_o, 0u, a.status);
+    if (!HF && ra.both && !mbar_wait(bar_o, 0u, a.status, a.wait_limit_other))
+      for (int cc = 0; cc < C; ++cc) tell_lost((unsigned)cc);
     if (C > 1) cluster_sync(); else __syncthreads();
-    const unsigned long long mine = lane < C ? S.best[lane] : ~0ull;
+    const unsigned long long mine = lane < C || lane == kResMaxCluster ? S.best[lane] : ~0ull;
     const unsigned long long b = warp_min_u64(mine);
+    if (b == kLostBest) return leave_unit();
     if (HF) {  // positions are distinct: one CTA has it
       const unsigned who = __ballot_sync(kFull, mine == b && lane < C);
       e_first = max(0, min(S.best_slot[__ffs(who) - 1], n - 1));
@@ -814,6 +850,7 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
         S.kmin[0] = mn;
         S.kmax[0] = mx;
       }
+      if (S.lost) tell_lost((unsigned)tid);
     }
     if (C > 1) {  // this slice's keys to every peer (the tail of the last slice carries padding)
       const int q4 = (R + 3) >> 2;
@@ -828,10 +865,12 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
         }
       }
     }
-    if (!HF && ra.both) mbar_wait(bar_o, 0u, a.status);
+    if (!HF && ra.both && !mbar_wait(bar_o, 0u, a.status, a.wait_limit_other))
+      for (int cc = 0; cc < C; ++cc) tell_lost((unsigned)cc);
     if (C > 1) cluster_sync(); else __syncthreads();
     kmin = __reduce_min_sync(kFull, lane < C ? S.kmin[lane] : 0xffffffffu);
-    kmax = __reduce_max_sync(kFull, lane < C ? S.kmax[lane] : 0u);
+    kmax = __reduce_max_sync(kFull, lane < C || lane == kResMaxCluster ? S.kmax[lane] : 0u);
+    if (kmax == kLostKey) return leave_unit();
     Selection sel = resident_select(
         [&](auto use) {  // four keys per load
           const int nv = n >> 2;
@@ -1135,14 +1174,22 @@ __global__ void __launch_bounds__(kThreads, 3) resident_evict_kernel(const Resid
     }
   }
   if (!ra.both) {
-    mbar_wait(bar_o, 0u, a.status);
+    // The scored tensor is compacted: a wait that gives up here leaves the other
+    // one's rows as they are, and the unit's contents are unspecified.  Its copy
+    // lands before the barrier, after which peers write what it reads.
+    const bool landed = mbar_wait(bar_o, 0u, a.status, a.wait_limit_other);
+    if (!landed) {
+      mbar_wait(bar_o, 0u, a.status, kWaitLimit);
+      __threadfence();  // the status first
+      a.len[seq] = mark_len(len0);
+    }
     // every CTA holds its rows of the other tensor, and has read its peers'
     // partial results
     if (C > 1) {
       cluster_arrive_relaxed();
       cluster_wait();
     }
-    write_rows(ob, L.obuf);
+    if (landed) write_rows(ob, L.obuf);
   } else {
     const bool late = C > 1 && (exchange || disp);
     if (late) cluster_arrive_relaxed();

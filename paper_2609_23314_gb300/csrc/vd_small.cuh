@@ -55,6 +55,8 @@ struct SmallSmem {
   float fsh[kWarps];
   float inv_mnorm;
   int mu_zero;
+  int lost;               // a wait for this unit's rows gave up
+  uint32_t any_lost;      // rank 0: a unit of the sequence did (set by its CTA)
 };
 
 struct SmallLayout {
@@ -123,7 +125,11 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
     mbar_init(bar_v, 1);
     mbar_init(bar_k, 1);
     fence_mbar_init();
+    S.lost = 0;
+    S.any_lost = 0u;
   }
+  const int C = a.cluster;
+  if (sa.set_len && C > 1) cluster_arrive();  // waited for before peers set any_lost
   grid_dependency_wait();
   grid_launch_dependents();
   const int d = a.d, d8 = d >> 3, cap = a.capacity;
@@ -133,7 +139,6 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
   uint32_t* keys = reinterpret_cast<uint32_t*>(smem_raw + L.keys);
   uint16_t* perm = reinterpret_cast<uint16_t*>(smem_raw + L.perm);
   const int tid = threadIdx.x, lane = tid & 31;
-  const int C = a.cluster;
   const unsigned rank = C > 1 ? cluster_ctarank() : 0u;
   const int u = (int)blockIdx.x;
   // a CTA past the last unit (impossible for the host's grid) reads and
@@ -186,22 +191,26 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
     const double rs_old = rsu && tid < d ? rsu[tid] : 0.0;
     const double dn = (double)n, rn = tid < d ? 1.0 / dn : 0.0;
     __syncthreads();
-    mbar_wait(bar_v, 0u, a.status);
+    // a wait that gives up leaves the unit as it is: what follows computes on
+    // whatever the buffers hold (every index is clamped) and stores none of it
+    if (!mbar_wait(bar_v, 0u, a.status, a.wait_limit)) S.lost = 1;
     auto vrow = [&](int r) { return Vs + (size_t)r * d; };
 
     if (!evict) {
       // ---- nothing to evict: append (fused), running sum += appended rows --
-      mbar_wait(bar_k, 0u, a.status);
-      if (FUSED)
+      if (!mbar_wait(bar_k, 0u, a.status, a.wait_limit_other)) S.lost = 1;
+      __syncthreads();
+      const bool landed = S.lost == 0;
+      if (FUSED && landed)
         for (int c = tid; c < a.B * d8; c += kThreads) {
           const int r = len0 + c / d8, col = (c % d8) * 8;
           st16(kb + (size_t)r * d + col, ld_shared16(ks_a + (uint32_t)(r * d + col) * 2u));
           st16(vb + (size_t)r * d + col, ld_shared16(vs_a + (uint32_t)(r * d + col) * 2u));
         }
-      if (a.kept_out)
+      if (a.kept_out && landed)
         for (int i = tid; i < a.N; i += kThreads) a.kept_out[(size_t)u * a.N + i] = i < n ? i : -1;
-      if (DECODE && a.evicted_out && tid == 0) a.evicted_out[u] = -1;
-      if (rsu && a.B > 0) {
+      if (DECODE && a.evicted_out && landed && tid == 0) a.evicted_out[u] = -1;
+      if (rsu && a.B > 0 && landed) {
         const ff t = small_column_sum(d, a.B, [&](int i) { return vrow(first_new + i); },
                                       [](int) { return 1.f; }, S);
         if (tid < d) rsu[tid] = rs_old + (double)t.hi + (double)t.lo;
@@ -308,27 +317,31 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
         return min((int)perm[i], n - 1);
       };
 
-      // ---- outputs --------------------------------------------------------
-      if (a.kept_out)
-        for (int i = tid; i < a.N; i += kThreads)
-          a.kept_out[(size_t)u * a.N + i] = i < Nb ? slot(i) : -1;
-      if (DECODE && a.evicted_out && tid == 0) a.evicted_out[u] = e_first;
-
       // ---- 5. running sum: (S + appended) - evicted rows ------------------
+      double s_left = s_app;
       if (rsu) {
         const ff t = small_column_sum(d, n - Nb, [&](int i) { return vrow(slot(Nb + i)); },
                                       [](int) { return -1.f; }, S);
-        if (tid < d) rsu[tid] = s_app + (double)t.hi + (double)t.lo;
+        if (tid < d) s_left = s_app + (double)t.hi + (double)t.lo;
       }
+
+      // ---- outputs, once K has landed too --------------------------------
+      if (!mbar_wait(bar_k, 0u, a.status, a.wait_limit_other)) S.lost = 1;
+      __syncthreads();
+      const bool landed = S.lost == 0;
+      if (rsu && landed && tid < d) rsu[tid] = s_left;
+      if (a.kept_out && landed)
+        for (int i = tid; i < a.N; i += kThreads)
+          a.kept_out[(size_t)u * a.N + i] = i < Nb ? slot(i) : -1;
+      if (DECODE && a.evicted_out && landed && tid == 0) a.evicted_out[u] = e_first;
 
       // ---- 6. compaction from the shared-memory copy ---------------------
       // (fused: the kept new rows below the budget are written too)
       const int r_begin = FUSED ? min(e_first, len0) : e_first;
-      mbar_wait(bar_k, 0u, a.status);
       const int ci = lane & (a.lpr - 1), g = tid / a.lpr, ng = kThreads / a.lpr;
       const unsigned char* vp = reinterpret_cast<const unsigned char*>(Vs) + ci * 16;
       const unsigned char* kp = reinterpret_cast<const unsigned char*>(Ks) + ci * 16;
-      if (ci < d8)
+      if (ci < d8 && landed)
         for (int r0 = r_begin + g; r0 < Nb; r0 += 2 * ng) {
           uint4 qk[2], qv[2];  // two rows of each tensor in flight
 #pragma unroll
@@ -346,12 +359,27 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
           }
         }
     }
+    if (tid == 0 && S.lost) {
+      mbar_wait(bar_v, 0u, a.status, kWaitLimit);
+      mbar_wait(bar_k, 0u, a.status, kWaitLimit);
+      if (!sa.set_len) {
+        __threadfence();  // the status first
+        a.len[seq] = mark_len(len0);
+      }
+    }
   }
 
   // ---- the sequence's new length, once every unit of it has read len -----
   if (!sa.set_len) return;  // a launch of its own does it
-  if (C > 1) cluster_sync(); else __syncthreads();
-  if (ok && (evict || FUSED) && rank == 0 && tid == 0 && u + C <= sa.n_units)
+  if (C > 1) {
+    cluster_wait();  // every CTA has set up its shared memory (long ago)
+    if (ok && tid == 0 && S.lost) st_cluster_u32(mapa(smem_addr(&S.any_lost), 0u), 1u);
+    cluster_sync();
+  } else {
+    if (tid == 0 && S.lost) S.any_lost = 1u;
+    __syncthreads();
+  }
+  if (ok && (evict || FUSED) && rank == 0 && tid == 0 && u + C <= sa.n_units && !S.any_lost)
     a.len[seq] = evict ? Nb : n;
 }
 
