@@ -132,29 +132,77 @@ __global__ void __launch_bounds__(kThreads) vd_rsum_init_kernel(const uint16_t* 
 // ---------------------------------------------------------------------------
 namespace {
 
-// A cluster-size decision for one launch shape (the occupancy queries behind
-// it cost more host time than a small eviction takes on the device).
-struct ClusterChoice {
-  const void* kern;
-  long long units;
-  int d, capacity, kind, want, c;  // kind: vd::kKind*, or kFitsKind (cached_fits)
-  size_t smem;
-  long long solo, want_solo;       // split launch: units run one CTA each (split_plan)
+// How calls of one shape are launched.  The occupancy queries behind it, up to
+// two dozen, take 2.3 us of host time (a call 8.3 us through the Python binding,
+// 6.1 with its plan at hand), as much as a small eviction's phases take on the
+// device: so the answers are kept.
+struct PlanKey {
+  const void* kern;           // the streaming kernel; fits plans: the short-cache kernel
+  long long units, want_solo;
+  int d, capacity, kind, running, want_cluster, want_resident;
+  bool operator==(const PlanKey& o) const {
+    return kern == o.kern && units == o.units && want_solo == o.want_solo && d == o.d &&
+           capacity == o.capacity && kind == o.kind && running == o.running &&
+           want_cluster == o.want_cluster && want_resident == o.want_resident;
+  }
 };
-constexpr int kChoiceSlots = 32;
+struct Plan {
+  int cluster;          // fits plans: 0 if the cluster does not fit
+  bool resident, both;  // the resident kernel; with a buffer for each tensor
+  size_t smem;
+  long long solo;       // split launch: units run one CTA each (split_plan)
+};
+// 1024 shapes per device, in sets of 4 picked by the key's hash: a program that
+// serves a few hundred batch sizes with a few kinds of calls finds them all again.
+constexpr int kPlanSets = 256, kPlanWays = 4;
+struct PlanSet {
+  PlanKey key[kPlanWays];
+  Plan plan[kPlanWays];
+  int used, next;  // entries in use; the one replaced next
+};
 
 struct DeviceState {
   bool ready = false;
   unsigned* status = nullptr;
   int sms = 0;
   int smem_optin = 0;
-  ClusterChoice choice[kChoiceSlots];  // guarded by g_mu; replaced round-robin
-  int n_choice = 0, next_choice = 0;
+  int smem_sm = 0, smem_reserved = 0;  // per SM; what each CTA takes of it besides its own
+  PlanSet plans[kPlanSets];            // guarded by g_mu
 };
 
 constexpr int kMaxDevices = 64;
 std::mutex g_mu;
 DeviceState g_dev[kMaxDevices];
+
+PlanSet& plan_set(DeviceState& st, const PlanKey& k) {
+  unsigned long long h = reinterpret_cast<uintptr_t>(k.kern);
+  for (const long long x : {k.units, k.want_solo, (long long)k.d, (long long)k.capacity,
+                            (long long)k.kind, (long long)k.running, (long long)k.want_cluster,
+                            (long long)k.want_resident})
+    h = (h ^ (unsigned long long)x) * 0x9e3779b97f4a7c15ull, h ^= h >> 29;
+  return st.plans[h % kPlanSets];
+}
+
+bool find_plan(DeviceState& st, const PlanKey& k, Plan* out) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  const PlanSet& s = plan_set(st, k);
+  for (int i = 0; i < s.used; ++i)
+    if (s.key[i] == k) {
+      *out = s.plan[i];
+      return true;
+    }
+  return false;
+}
+
+void keep_plan(DeviceState& st, const PlanKey& k, const Plan& p) {
+  std::lock_guard<std::mutex> lk(g_mu);
+  PlanSet& s = plan_set(st, k);
+  const int i = s.next;
+  s.key[i] = k;
+  s.plan[i] = p;
+  s.next = (i + 1) % kPlanWays;
+  if (s.used < kPlanWays) ++s.used;
+}
 
 // general: the score pass for any rule and head dim, else the batched one
 // (vd::batched_scores)
@@ -210,6 +258,8 @@ vd_status device_state(DeviceState** out) {
     st.status = static_cast<unsigned*>(ptr);
     st.sms = p.multiProcessorCount;
     st.smem_optin = (int)p.sharedMemPerBlockOptin;
+    st.smem_sm = (int)p.sharedMemPerMultiprocessor;
+    st.smem_reserved = (int)p.reservedSharedMemPerBlock;
     if (cudaFuncSetAttribute(reinterpret_cast<const void*>(&vd_rsum_init_kernel),
                              cudaFuncAttributeMaxDynamicSharedMemorySize,
                              st.smem_optin) != cudaSuccess)
@@ -475,59 +525,29 @@ long long split_plan(const void* kern, long long units, int d, int capacity, int
   return best_solo;
 }
 
-// choose_cluster (and split_plan), remembered per launch shape.  A forced
-// cluster size (VD_CLUSTER_SIZE) turns the automatic split off;
-// VD_SOLO_UNITS with it forces a split whose first launch runs that many
-// units (at most all but one) one CTA each, for tests.
-int cached_cluster(const void* kern, long long units, int d, int capacity, int kind,
-                   bool holefill, bool heavy, bool resum, DeviceState& st, size_t* smem_out, long long* solo_out) {
-  const int key = kind | (resum ? 256 : 0);  // of the remembered choice
-  const char* env = std::getenv("VD_CLUSTER_SIZE");
-  const int want = env ? std::atoi(env) : 0;
-  // want_solo: the forced first part (VD_SOLO_UNITS, with a forced cluster
-  // size), else 0 when the split is turned off, else -1 (automatic)
-  long long want_solo = -1;
-  if (want >= 1) {
-    const char* senv = std::getenv("VD_SOLO_UNITS");
-    if (senv) want_solo = std::atoll(senv);
-  } else {
-    const char* off = std::getenv("VD_SPLIT_LAUNCH");
-    if (off && std::atoi(off) == 0) want_solo = 0;
-  }
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    for (int i = 0; i < st.n_choice; ++i) {
-      const ClusterChoice& e = st.choice[i];
-      if (e.kern == kern && e.units == units && e.d == d && e.capacity == capacity &&
-          e.kind == key && e.want == want && e.want_solo == want_solo) {
-        *smem_out = e.smem;
-        *solo_out = e.solo;
-        return e.c;
-      }
+// choose_cluster and split_plan.  A forced cluster size (VD_CLUSTER_SIZE) turns
+// the automatic split off; VD_SOLO_UNITS with it forces a split whose first
+// launch runs that many units (at most all but one) one CTA each, for tests
+// (want_solo: that, else 0 when VD_SPLIT_LAUNCH turns the split off, else -1).
+Plan streaming_plan(const PlanKey& k, bool holefill, bool heavy, bool resum,
+                    const DeviceState& st) {
+  Plan p{};
+  p.cluster = choose_cluster(k.kern, k.units, k.d, k.capacity, k.kind, holefill, heavy, resum,
+                             k.want_cluster, st, &p.smem);
+  if (k.want_cluster >= 1 && k.want_solo > 0) {
+    p.solo = std::min(k.want_solo, k.units - 1);
+  } else if (k.want_cluster < 1 && k.want_solo != 0 &&
+             ((k.kind == vd::kKindBlock && holefill) || k.kind == vd::kKindScore ||
+              k.kind == vd::kKindScoreBulk)) {
+    int c = p.cluster;
+    size_t smem = p.smem;
+    p.solo = split_plan(k.kern, k.units, k.d, k.capacity, k.kind, st, &c, &smem);
+    if (p.solo > 0) {
+      p.cluster = c;
+      p.smem = smem;
     }
   }
-  int c = choose_cluster(kern, units, d, capacity, kind, holefill, heavy, resum, want, st, smem_out);
-  long long solo = 0;
-  if (want >= 1 && want_solo > 0) {
-    solo = std::min(want_solo, units - 1);
-  } else if (want < 1 && want_solo != 0 &&
-             ((kind == vd::kKindBlock && holefill) || kind == vd::kKindScore ||
-              kind == vd::kKindScoreBulk)) {
-    int cs = c;
-    size_t sm = *smem_out;
-    solo = split_plan(kern, units, d, capacity, kind, st, &cs, &sm);
-    if (solo > 0) {
-      c = cs;
-      *smem_out = sm;
-    }
-  }
-  std::lock_guard<std::mutex> lk(g_mu);
-  st.choice[st.next_choice] =
-      ClusterChoice{kern, units, d, capacity, key, want, c, *smem_out, solo, want_solo};
-  st.next_choice = (st.next_choice + 1) % kChoiceSlots;
-  if (st.n_choice < kChoiceSlots) ++st.n_choice;
-  *solo_out = solo;
-  return c;
+  return p;
 }
 
 // The short-cache kernel (vd_small.cuh) takes a block or decode event when
@@ -551,30 +571,16 @@ bool use_small(const vd_cache* c, bool score_only, bool holefill, const float* d
   return vd::small_layout(c->capacity, c->head_dim).total <= (size_t)st.smem_optin;
 }
 
-// groups clusters of c CTAs: the fused kernel's grid is units x c CTAs (a
-// cluster per unit), the short-cache kernel's n_seq x units_per_seq (a
-// cluster per sequence, a CTA per unit)
-// cluster_fits, remembered per launch shape (the occupancy query costs
-// several microseconds of host time, as much as a short-cache event takes on
-// the device); entries are marked kind == kFitsKind in the choice cache.
-constexpr int kFitsKind = 3;
+// cluster_fits, kept like the plans (of kind kFitsKind).
+constexpr int kFitsKind = -1;
 bool cached_fits(const void* kern, long long groups, int c, size_t smem, DeviceState& st) {
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    for (int i = 0; i < st.n_choice; ++i) {
-      const ClusterChoice& e = st.choice[i];
-      if (e.kern == kern && e.units == groups && e.kind == kFitsKind && e.want == c &&
-          e.smem == smem)
-        return e.c != 0;
-    }
+  const PlanKey k{kern, groups, (long long)smem, 0, 0, kFitsKind, 0, c, 0};
+  Plan p{};
+  if (!find_plan(st, k, &p)) {
+    p.cluster = cluster_fits(kern, groups, c, smem, st) ? c : 0;
+    keep_plan(st, k, p);
   }
-  const bool fits = cluster_fits(kern, groups, c, smem, st);
-  std::lock_guard<std::mutex> lk(g_mu);
-  st.choice[st.next_choice] =
-      ClusterChoice{kern, groups, 0, 0, kFitsKind, c, fits ? c : 0, smem, 0, 0};
-  st.next_choice = (st.next_choice + 1) % kChoiceSlots;
-  if (st.n_choice < kChoiceSlots) ++st.n_choice;
-  return fits;
+  return p.cluster != 0;
 }
 
 // A plain kernel of kThreads-thread blocks as a programmatic dependent launch
@@ -598,6 +604,9 @@ vd_status launch_dependent(unsigned blocks, cudaStream_t s, void (*kern)(Params.
   return VD_OK;
 }
 
+// groups clusters of c CTAs: the streaming and resident kernels' grids are units x
+// c CTAs (a cluster per unit), the short-cache kernel's n_seq x units_per_seq (a
+// cluster per sequence, a CTA per unit) or units x 1.
 vd_status launch(const void* kern, long long groups, int c, size_t smem, const void* params,
                  cudaStream_t s, bool dependent = false) {
   cudaLaunchConfig_t cfg = {};
@@ -646,61 +655,49 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
 // units 39.1 / 20.1; hole-fill decode, 4097 rows, 8 units 19.2 / 11.0, 201 rows,
 // 4800 units 138 / 86.  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
 // c CTAs (100 + c: with both buffers), for tests.  Returns C, or 0.
-constexpr int kResidentKind = 4;  // and 5: with the running mean
 constexpr int kResidentMinRows = 64;
 
-int resident_plan(const void* kern, long long units, int d, int capacity, bool decode,
-                  bool holefill, bool running, DeviceState& st, size_t* smem_out, bool* both_out) {
-  const char* env = std::getenv("VD_RESIDENT");
-  const int want = env ? std::atoi(env) : -1;
-  if (want == 0 || std::getenv("VD_CLUSTER_SIZE") || capacity > vd::kMaxMarkedLen) return 0;
-  const int kind = kResidentKind + (running ? 1 : 0);
-  {
-    std::lock_guard<std::mutex> lk(g_mu);
-    for (int i = 0; i < st.n_choice; ++i) {
-      const ClusterChoice& e = st.choice[i];
-      if (e.kern == kern && e.units == units && e.d == d && e.capacity == capacity &&
-          e.kind == kind && e.want == want) {
-        *smem_out = e.smem;
-        *both_out = e.solo != 0;
-        return e.c;
-      }
-    }
-  }
+int resident_plan(const void* kern, const PlanKey& k, bool decode, bool holefill,
+                  const DeviceState& st, size_t* smem_out, bool* both_out) {
+  const int want = k.want_resident, capacity = k.capacity;
+  const long long units = k.units;
+  if (want == 0 || capacity > vd::kMaxMarkedLen) return 0;
   auto smem_of = [&](int c, bool both) {
-    return vd::resident_layout(capacity, d, c, decode, holefill, running, both).total;
+    return vd::resident_layout(capacity, k.d, c, decode, holefill, k.running != 0, both).total;
   };
-  // units that run at once on clusters of c CTAs
-  auto at_once = [&](int c, bool both) -> long long {
+  // whether `need` units run at once on clusters of c CTAs (asked only where
+  // their shared memory alone lets them)
+  auto at_once = [&](int c, bool both, long long need) {
     const size_t smem = smem_of(c, both);
-    return smem > (size_t)st.smem_optin ? 0 : active_clusters(kern, units, c, smem, st);
+    if (smem > (size_t)st.smem_optin) return false;
+    const long long ctas = (long long)st.sms * (st.smem_sm / ((int)smem + st.smem_reserved));
+    return ctas / c >= need && active_clusters(kern, units, c, smem, st) >= need;
   };
   int c = 0;
   bool both = false;
   if (want > 0) {
     c = want % 100;
     both = want >= 100 && !holefill;
-    if (c < 1 || c > vd::kResMaxCluster || at_once(c, both) < 1) c = 0;
+    if (c < 1 || c > vd::kResMaxCluster || !at_once(c, both, 1)) c = 0;
   } else {
     const long long room = (decode ? 3LL : 2LL) * st.sms;
     if (units <= room) {
       const long long most = std::min<long long>(room / units, capacity / kResidentMinRows);
       for (c = (int)std::max(1LL, std::min(12LL, most)); c >= 1; --c)
-        if (at_once(c, false) >= units) break;
-      both = !holefill && c >= 1 && at_once(c, true) >= units;
+        if (at_once(c, false, units)) break;
+      both = !holefill && c >= 1 && at_once(c, true, units);
     }
-    if (holefill && !decode && c > 1 && units * capacity * d * 2 > 12LL << 20) c = 0;
-    if (c < 1 && at_once(1, false) >= (decode ? 2LL : 3LL) * st.sms) c = 1;
+    if (holefill && !decode && c > 1 && units * capacity * k.d * 2 > 12LL << 20) c = 0;
+    if (c < 1 && at_once(1, false, (decode ? 2LL : 3LL) * st.sms)) c = 1;
   }
-  const size_t smem = c >= 1 ? smem_of(c, both) : 0;
-  std::lock_guard<std::mutex> lk(g_mu);
-  st.choice[st.next_choice] =
-      ClusterChoice{kern, units, d, capacity, kind, want, c, smem, both ? 1 : 0, 0};
-  st.next_choice = (st.next_choice + 1) % kChoiceSlots;
-  if (st.n_choice < kChoiceSlots) ++st.n_choice;
-  *smem_out = smem;
+  *smem_out = c >= 1 ? smem_of(c, both) : 0;
   *both_out = both;
   return c;
+}
+
+int env_int(const char* name, int unset) {
+  const char* s = std::getenv(name);
+  return s ? std::atoi(s) : unset;
 }
 
 // Polls after which a device wait gives up.  VD_WAIT_LIMIT=a or a:b lowers them,
@@ -756,6 +753,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     return VD_ERR_UNSUPPORTED;
   const void* kern = score_only ? score_kernel(var, general)
                                 : evict_kernel(var, decode, holefill, fused, general);
+  const void* rk = score_only ? nullptr : resident_kernel(var, decode, holefill, fused);
   const long long units = (long long)c->n_seq * c->n_layer * c->n_kv_head;
 
   vd::EvictArgs a;
@@ -809,22 +807,35 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     r = launch(sk, units, 1, ssmem, &sa, s, true);
     return r != VD_OK ? r : clamp_lengths();
   }
-  size_t smem = 0;
-  long long solo = 0;
-  if (!score_only) {
-    const void* rk = resident_kernel(var, decode, holefill, fused);
+  const bool cluster_env = std::getenv("VD_CLUSTER_SIZE") != nullptr;
+  const int want_cluster = env_int("VD_CLUSTER_SIZE", 0);
+  long long want_solo = -1;  // see streaming_plan
+  if (want_cluster >= 1)
+    want_solo = env_int("VD_SOLO_UNITS", -1);
+  else if (env_int("VD_SPLIT_LAUNCH", 1) == 0)
+    want_solo = 0;
+  // a forced cluster size is one of the streaming kernel's
+  const int want_resident = score_only || cluster_env ? 0 : env_int("VD_RESIDENT", -1);
+  const PlanKey key{kern, units, want_solo, c->head_dim, c->capacity, kind,
+                    mu == VD_MU_RUNNING ? 1 : 0, want_cluster, want_resident};
+  Plan plan{};
+  if (!find_plan(*st, key, &plan)) {
+    size_t rsmem = 0;
     bool both = false;
-    a.cluster = resident_plan(rk, units, c->head_dim, c->capacity, decode, holefill,
-                              mu == VD_MU_RUNNING, *st, &smem, &both);
-    if (a.cluster > 0) {
-      const vd::ResidentArgs ra{a, both ? 1 : 0};
-      r = launch(rk, units, a.cluster, smem, &ra, s, true);
-      return r != VD_OK ? r : clamp_lengths();
-    }
+    const int rc = resident_plan(rk, key, decode, holefill, *st, &rsmem, &both);
+    plan = rc > 0 ? Plan{rc, true, both, rsmem, 0}
+                  : streaming_plan(key, holefill, general,
+                                   mu == VD_MU_RECOMPUTE && var != VD_SCORE_NORM, *st);
+    keep_plan(*st, key, plan);
   }
-  a.cluster =
-      cached_cluster(kern, units, c->head_dim, c->capacity, kind, holefill, general,
-                     mu == VD_MU_RECOMPUTE && var != VD_SCORE_NORM, *st, &smem, &solo);
+  a.cluster = plan.cluster;
+  const size_t smem = plan.smem;
+  if (plan.resident) {
+    const vd::ResidentArgs ra{a, plan.both ? 1 : 0};
+    r = launch(rk, units, a.cluster, smem, &ra, s, true);
+    return r != VD_OK ? r : clamp_lengths();
+  }
+  const long long solo = plan.solo;
   if (smem > (size_t)st->smem_optin) return VD_ERR_UNSUPPORTED;
 
   if (solo > 0) {
