@@ -19,6 +19,16 @@ def orc():
     return oracle.load()
 
 
+@pytest.fixture(params=["automatic", "streaming"])
+def kernel_route(request, monkeypatch):
+    """Runs a test with the kernel the library picks for its shapes, which for
+    small ones is the short-cache or the resident kernel, and again with the
+    streaming kernel, which the large workloads take."""
+    if request.param == "streaming":
+        monkeypatch.setenv("VD_SMALL_PATH", "0")
+        monkeypatch.setenv("VD_RESIDENT", "0")
+
+
 def pytest_terminal_summary(terminalreporter):
     """The worst score error each GPU test saw against the oracle, per rule:
     relative (over scores above 1e-6) and as a fraction of the tolerance."""

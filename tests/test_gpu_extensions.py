@@ -147,6 +147,7 @@ def test_negative_zero_weight_and_nan_rank(orc, var, cluster, monkeypatch):
         assert np.all(sh[u, 0:40:2] == 0.0)
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_uniform_attention_keeps_the_valuediff_set(orc):
     """App. A: with a_j = 1/n the weighted rule ranks like ValueDiff."""
     d, N, n = 128, 150, 200

@@ -95,6 +95,7 @@ def assert_same(a, b):
         assert torch.equal(rsa, rsb)
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 @pytest.mark.parametrize("d", [64, 128, 200, 256])
 @pytest.mark.parametrize("mu", [vd.VD_MU_RECOMPUTE, vd.VD_MU_RUNNING], ids=["recompute", "running"])
@@ -192,6 +193,7 @@ def run_both_holefill(cache, k_new, v_new, B, N, var, mu, lens):
     return out
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 @pytest.mark.parametrize("mu", [vd.VD_MU_RECOMPUTE, vd.VD_MU_RUNNING], ids=["recompute", "running"])
 @pytest.mark.parametrize("d", [128, 200])
@@ -212,6 +214,7 @@ def test_fused_holefill_equals_append_then_evict(var, mu, d):
             assert torch.equal(pa[u, :n], pb[u, :n]), u
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_fused_holefill_repeated_events():
     """Five hole-fill block events in a row at the benchmark's head dim, fused
     and two-call, stay identical (positions and running mean carried along)."""
@@ -244,6 +247,7 @@ def test_fused_holefill_repeated_events():
         assert torch.equal(pa[..., :N], pb[..., :N]) and torch.equal(rsa, rsb)
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 @pytest.mark.parametrize("mu", [vd.VD_MU_RECOMPUTE, vd.VD_MU_RUNNING], ids=["recompute", "running"])
 @pytest.mark.parametrize("layout", ["ordered", "holefill"])
@@ -308,6 +312,7 @@ def test_fused_decode_steps(var, mu, layout):
     assert ca.len.cpu().tolist() == [N, N]
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_fused_per_sequence_budgets():
     """Per-sequence budgets (N_dev): block and decode steps, fused against the
     two-call path, including a sequence whose budget lies below its length."""
@@ -352,6 +357,7 @@ def test_fused_per_sequence_budgets():
         assert torch.equal(units_view(ca.v)[u, :n].view(torch.int16), units_view(cb.v)[u, :n].view(torch.int16))
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 @pytest.mark.parametrize("keys", [False, True], ids=["values", "keys"])
 @pytest.mark.parametrize("weighted", [False, True], ids=["plain", "weighted"])

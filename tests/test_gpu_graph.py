@@ -2,15 +2,19 @@
 same calls run eagerly: the block and decode evictions (whose length update
 is a programmatic dependent launch), the hole-fill and score-only calls at
 sizes that take the split launch (two launches, the second a programmatic
-dependent of the first), and the short-cache kernel.  Needs a GB300."""
+dependent of the first), and the short-cache kernel; each with the kernel that
+the library picks (the resident one for all evictions but the last) and with
+the streaming kernel.  Needs a GB300."""
 from __future__ import annotations
+
+import os
 
 import pytest
 import torch
 
 import paper_2609_23314_gb300 as vd
 from paper_2609_23314_gb300 import build, workloads as wl
-from vd_gpu import new_cache, units_view
+from vd_gpu import evictions, new_cache, units_view
 
 pytestmark = pytest.mark.gpu
 
@@ -74,13 +78,15 @@ def call(kind, s, N, B):
 CASES = {
     # kind: (n_seq, layers, heads, capacity, d, lens, N, B)
     "ordered_block": (2, 3, 4, 640, 128, [512, 500], 512, 128),
-    "holefill_block": (1, 20, 8, 320, 128, [256], 256, 64),        # 160 units: split launch
+    "holefill_block": (1, 20, 8, 320, 128, [256], 256, 64),        # 160 units
     "decode": (3, 4, 4, 1025, 128, [1024, 1024, 1000], 1024, 1),
-    "score": (1, 21, 8, 700, 256, [697], 1, 0),                     # 168 units: split launch
+    "score": (1, 21, 8, 700, 256, [697], 1, 0),                     # 168 units
     "short_cache": (1, 1, 2, 160, 64, [128], 128, 32),              # the short-cache kernel
 }
+SPLIT = {"holefill_block", "score"}  # two launches of the streaming kernel
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("kind", list(CASES))
 def test_graph_replay_matches_eager(kind):
     n_seq, L, H, cap, d, lens, N, B = CASES[kind]
@@ -94,6 +100,11 @@ def test_graph_replay_matches_eager(kind):
     # the plan for this shape is cached by the eager call; capture on static
     # buffers, put the initial state back, replay once
     static = clone(base)
+    took = [k for k, _ in evictions(lambda: call(how, static, N, B))]
+    if os.environ.get("VD_RESIDENT") == "0" or kind == "score":
+        assert took == ["evict_kernel"] * (2 if kind in SPLIT else 1)
+    else:
+        assert took == ["small_evict_kernel" if kind == "short_cache" else "resident_evict_kernel"]
     side = torch.cuda.Stream()
     side.wait_stream(torch.cuda.current_stream())
     with torch.cuda.stream(side):

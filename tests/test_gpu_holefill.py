@@ -125,6 +125,7 @@ def test_holefill_block_event(orc, var, cluster, monkeypatch):
     run_event(orc, var, cache, pos, pos_new, N, B, vd.VD_MU_RECOMPUTE, None)
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 def test_holefill_prefill_trajectory_running(orc, var):
     """Block prompt processing in the hole-fill layout with the running mean:
@@ -147,6 +148,7 @@ def test_holefill_prefill_trajectory_running(orc, var):
     assert torch.max(torch.abs(ref - rs)).item() <= 1e-9
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 def test_holefill_decode_steps(orc, var):
     d, N = 64, 96
@@ -166,6 +168,7 @@ def test_holefill_decode_steps(orc, var):
     assert torch.max(torch.abs(ref - rs)).item() <= 1e-9
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 def test_holefill_ties_break_by_position(orc, var):
     """Exact ties (duplicates, small integers) with shuffled positions: the
@@ -181,6 +184,7 @@ def test_holefill_ties_break_by_position(orc, var):
         run_event(orc, var, cache, pos, pos_new, N, B, vd.VD_MU_RECOMPUTE, None)
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_holefill_per_sequence_budgets(orc):
     d, cap = 128, 400
     lens = [400, 390, 120, 3]
@@ -191,6 +195,7 @@ def test_holefill_per_sequence_budgets(orc):
     run_event(orc, oracle.L2, cache, pos, pos_new, 390, B, vd.VD_MU_RECOMPUTE, None, N_dev=Ns)
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_holefill_decode_moves_one_row():
     """A decode step in the hole-fill layout changes at most one slot below N
     and leaves every other row's bytes in place."""

@@ -166,6 +166,7 @@ def test_tiny_prefill_every_event(orc, var, mu):
 # ---------------------------------------------------------------------------
 # decode == block with B = 1, bit for bit
 # ---------------------------------------------------------------------------
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 def test_decode_equals_block_b1(var):
     d, N = 128, 300
@@ -216,6 +217,7 @@ def test_decode_steps_running_sum(orc, var):
 # block then decode events at head dims with the batched score pass (64, 256)
 # and without it (96), ragged batch tails, both mean modes
 # ---------------------------------------------------------------------------
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 @pytest.mark.parametrize("d", [64, 96, 256])
 @pytest.mark.parametrize("mu", [vd.VD_MU_RECOMPUTE, vd.VD_MU_RUNNING], ids=["recompute", "running"])
@@ -275,6 +277,7 @@ def test_all_rows_equal_keeps_first_n(var):
     assert int(cache.len[0]) == N
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("N", [1, 2, 499])
 def test_budget_extremes(orc, N):
     n, d = 500, 128
@@ -282,6 +285,7 @@ def test_budget_extremes(orc, N):
     evict_and_check(orc, cache, N, 0, oracle.L2, vd.VD_MU_RECOMPUTE)
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_poisoned_tail_never_read(orc):
     d, N, B, cap = 128, 100, 30, 200
     cache = filled_cache(2, 2, 2, cap, d, [N + B, N + B], seed=21)
@@ -299,6 +303,7 @@ def test_poisoned_tail_never_read(orc):
                        torch.full_like(cache.v[..., N + B:, :].view(torch.int16), 0x7FC0))
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_ragged_lengths_and_per_sequence_budgets(orc):
     d, cap = 128, 700
     lens = [700, 650, 100, 699, 3]
@@ -307,6 +312,7 @@ def test_ragged_lengths_and_per_sequence_budgets(orc):
     evict_and_check(orc, cache, 650, 0, oracle.L2, vd.VD_MU_RECOMPUTE, N_dev=Ns)
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_block_equals_one_shot_standard_eviction(orc):
     """B = T recovers standard eviction (Sec. 2.2): one event over the whole
     prompt equals the oracle's one-shot top-N."""

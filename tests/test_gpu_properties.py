@@ -52,6 +52,7 @@ def evict(cache, N, var):
     return kept.view(cache.units, N).cpu().numpy(), scores.view(cache.units, -1).cpu().numpy()
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARIANTS, ids=VAR_IDS)
 @pytest.mark.parametrize("factor", [2.0, 0.5])
 def test_positive_homogeneity(var, factor):
@@ -72,6 +73,7 @@ def test_positive_homogeneity(var, factor):
     assert np.array_equal(k1, k2)
 
 
+@pytest.mark.usefixtures("kernel_route")
 @pytest.mark.parametrize("var", VARIANTS, ids=VAR_IDS)
 def test_permutation_equivariance(var):
     """Shuffling the cached rows shuffles the scores with them and keeps the
@@ -95,6 +97,7 @@ def test_permutation_equivariance(var):
             assert np.all(near_tie_band(s1[u], N)[diff]), (u, diff[:8])
 
 
+@pytest.mark.usefixtures("kernel_route")
 def test_translation_invariance_of_l2():
     """v_j -> v_j + c for every j moves the mean by c and leaves every
     deviation v_j - mean unchanged.  With small-integer values and n a power

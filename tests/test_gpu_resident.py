@@ -18,9 +18,11 @@ import itertools
 import pytest
 import torch
 
+import oracle
 import paper_2609_23314_gb300 as vd
 from paper_2609_23314_gb300 import build, workloads as wl
-from vd_gpu import units_view
+from test_gpu_parity import evict_and_check, filled_cache
+from vd_gpu import evictions, units_view
 
 pytestmark = pytest.mark.gpu
 
@@ -80,36 +82,42 @@ def step(force, k, v, lens, N, B, var, mu, decode, fused, budgets, options, monk
         g = torch.Generator(device="cuda").manual_seed(3)
         attn = torch.rand(us + (cap,), generator=g, device="cuda") * 0.02
     pos = options["pos"].clone() if "pos" in options else None
+    out = dict(kept_idx_out=kept, scores_out=sc)
+    how = dict(N_dev=n_dev, variant=var, mu=mu, running_sum=rs)
     if pos is not None:
         first = torch.tensor([10 ** 6 + 1000 * s for s in range(n_seq)], dtype=torch.int32,
                              device="cuda")
-        hole = dict(pos=pos, pos_first_new=first)
+        how.update(pos=pos, pos_first_new=first)
+
+    def event():
         if decode and fused:
-            vd.vd_append_evict_decode(cache, *new, N, n_dev, var, mu, rs, ev, kept, sc, **hole)
+            vd.vd_append_evict_decode(cache, *new, N, evicted_out=ev, **how, **out)
+        elif decode and pos is not None:
+            vd.vd_evict_decode_holefill(cache, N, evicted_out=ev, **how, **out)
         elif decode:
-            vd.vd_evict_decode_holefill(cache, N, pos, first, n_dev, var, mu, rs, ev, kept, sc)
+            vd.vd_evict_decode(cache, N, evicted_out=ev, **how, **out)
+        elif pos is not None and not fused:
+            vd.vd_evict_block_holefill(cache, N, B=B, **how, **out)
+        elif options and pos is None:
+            call = vd.vd_append_evict_block_ex if fused else vd.vd_evict_block_ex
+            call(cache, *((*new, B) if fused else ()), N, **({} if fused else dict(B=B)),
+                 score_keys=keys, attn=attn, dispersion_out=sg, **how, **out)
         elif fused:
-            vd.vd_append_evict_block(cache, *new, B, N, n_dev, var, mu, rs, kept, sc, **hole)
+            vd.vd_append_evict_block(cache, *new, B, N, **how, **out)
         else:
-            vd.vd_evict_block_holefill(cache, N, pos, first, n_dev, B, var, mu, rs, kept, sc)
+            vd.vd_evict_block(cache, N, B=B, **how, **out)
+
+    took = evictions(event)  # a forced size that does not fit would run the streaming kernel
+    units = n_seq * L * H
+    if force == 0:
+        assert {k for k, _ in took} == {"evict_kernel"}
+    else:
+        assert took == [("resident_evict_kernel", units * (force % 100))], (force, took)
+    event()
+    if pos is not None:
         for s, m in enumerate(cache.len.tolist()):
             pos[s, ..., m:] = 0  # unspecified there
         sg = pos.float()
-    elif decode:
-        if fused:
-            vd.vd_append_evict_decode(cache, *new, N, n_dev, var, mu, rs, ev, kept, sc)
-        else:
-            vd.vd_evict_decode(cache, N, n_dev, var, mu, rs, ev, kept, sc)
-    elif options:
-        if fused:
-            vd.vd_append_evict_block_ex(cache, *new, B, N, n_dev, var, mu, rs, keys, attn, kept,
-                                        sc, sg)
-        else:
-            vd.vd_evict_block_ex(cache, N, n_dev, B, var, mu, rs, keys, attn, kept, sc, sg)
-    elif fused:
-        vd.vd_append_evict_block(cache, *new, B, N, n_dev, var, mu, rs, kept, sc)
-    else:
-        vd.vd_evict_block(cache, N, n_dev, B, var, mu, rs, kept, sc)
     status = vd.vd_get_device_status()
     return cache, rs, kept, ev, sc, sg, status
 
@@ -266,3 +274,54 @@ def test_rejected_lengths_leave_the_unit_alone(monkeypatch):
             assert vd.vd_get_device_status() == code
             assert int(cache.len[0]) == ln
             assert torch.equal(cache.v, v) and torch.equal(cache.k, k)
+
+
+# sequences, layers, KV heads, capacity, head dim -> CTAs per unit of the resident
+# kernel that the library picks by itself, or None for the streaming kernel
+AUTOMATIC = {
+    "long-rows": ((1, 1, 2, 1500, 128), 12),          # few units: the most CTAs per unit
+    "half-sms": ((1, 4, 19, 700, 128), 4),            # 76 units, 304 CTAs: two per SM
+    "two-per-sm": ((2, 4, 38, 200, 128), 1),          # 304 units: the last with one wave
+    "over-two-per-sm": ((2, 1, 153, 200, 128), 1),    # 306: three share an SM
+    "many-waves": ((3, 5, 80, 230, 96), 1),           # 1200 units
+    "too-large": ((2, 1, 153, 700, 128), None),       # one CTA per SM: the streaming kernel
+}
+
+
+@pytest.mark.parametrize("decode", [False, True], ids=["block", "decode"])
+@pytest.mark.parametrize("case", list(AUTOMATIC))
+def test_automatic_dispatch_matches_oracle(orc, case, decode, monkeypatch):
+    """The plans the library makes by itself, on both sides of the rule's lines
+    (for 152 SMs), against the fp64 oracle on a sample of the units."""
+    for name in ("VD_RESIDENT", "VD_SMALL_PATH", "VD_CLUSTER_SIZE"):
+        monkeypatch.delenv(name, raising=False)
+    (n_seq, L, H, cap, d), ctas = AUTOMATIC[case]
+    B = 1 if decode else 30
+    N = cap - B
+    cache = filled_cache(n_seq, L, H, cap, d, [cap] * n_seq, seed=cap)
+    units = cache.units
+    rs = torch.zeros(cache.unit_shape() + (d,), dtype=torch.float64, device="cuda")
+    cache.len.fill_(N)
+    vd.vd_running_sum_init(cache, rs)
+    cache.len.fill_(cap)
+
+    def event():
+        if decode:
+            vd.vd_evict_decode(cache, N, None, oracle.L2, RUN, rs)
+        else:
+            vd.vd_evict_block(cache, N, None, B, oracle.L2, RUN, rs)
+
+    took = evictions(event)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        if ctas is None:
+            assert {k for k, _ in took} == {"evict_kernel"}
+        elif decode and ctas > 1:  # decode: three CTAs per SM
+            assert took[0][0] == "resident_evict_kernel" and took[0][1] >= units * ctas
+        else:
+            assert took == [("resident_evict_kernel", units * ctas)], took
+    evict_and_check(orc, cache, N, B, oracle.L2, RUN, rs, units=range(0, units, max(1, units // 40)),
+                    decode=decode)
+    ref = torch.zeros_like(rs)
+    vd.vd_running_sum_init(cache, ref)
+    scale = units_view(cache.v).float().abs().sum(dim=1).max().item()
+    assert torch.max(torch.abs(ref - rs)).item() <= 1e-12 * scale

@@ -1,7 +1,7 @@
 """The short-cache kernel (one CTA per unit, the unit's rows in shared memory,
 one launch per event including the length update) against the fp64 oracle,
-step-locked, and against the fused kernel on the same inputs
-(VD_SMALL_PATH=0 forces the latter).  Needs a GB300."""
+step-locked, and against the streaming and the resident kernel on the same
+inputs (VD_SMALL_PATH=0 with VD_RESIDENT=0 or 1).  Needs a GB300."""
 from __future__ import annotations
 
 import numpy as np
@@ -12,7 +12,7 @@ import oracle
 import paper_2609_23314_gb300 as vd
 from paper_2609_23314_gb300 import build, workloads as wl
 from test_gpu_parity import evict_and_check, filled_cache
-from vd_gpu import bits, near_tie_band, units_view
+from vd_gpu import bits, evictions, near_tie_band, units_view
 
 pytestmark = pytest.mark.gpu
 
@@ -54,8 +54,9 @@ def check_running_sum(cache, rs):
 # ---------------------------------------------------------------------------
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 @pytest.mark.parametrize("mu", MUS, ids=MU_IDS)
-@pytest.mark.parametrize("shape", [(1, 1, 64, 160), (2, 3, 128, 120), (1, 16, 8, 700),
-                                   (3, 2, 24, 300)], ids=["1x1", "2x3", "1x16", "3x2"])
+@pytest.mark.parametrize("shape", [(1, 1, 64, 160), (2, 3, 128, 120), (1, 16, 8, 256),
+                                   (3, 2, 24, 250), (1, 16, 8, 700), (3, 2, 24, 300)],
+                         ids=["1x1", "2x3", "1x16", "3x2", "1x16-long", "3x2-long"])
 def test_block_event_matches_oracle(orc, var, mu, shape):
     L, H, d, cap = shape
     N, B = cap * 2 // 3, cap // 3
@@ -138,21 +139,34 @@ def test_fused_append_matches_two_calls(var, mu, decode):
 
 
 # ---------------------------------------------------------------------------
-# the same event through the fused kernel: same kept sets outside near ties,
-# same compacted rows where the sets agree, scores within the tolerance
+# the same event through the streaming and the resident kernel: same kept sets
+# outside near ties, same compacted rows where the sets agree, scores within the
+# tolerance
 # ---------------------------------------------------------------------------
+def on_kernel(kernel, monkeypatch):
+    """Makes the calls that follow take the named kernel."""
+    monkeypatch.setenv("VD_SMALL_PATH", "1" if kernel == "small_evict_kernel" else "0")
+    monkeypatch.setenv("VD_RESIDENT", "1" if kernel == "resident_evict_kernel" else "0")
+
+
+@pytest.mark.parametrize("other", ["evict_kernel", "resident_evict_kernel"])
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
-def test_agrees_with_the_fused_kernel(orc, var, monkeypatch):
+def test_agrees_with_the_fused_kernel(orc, var, other, monkeypatch):
     d, N, B = 64, 100, 40
     lens = [N + B, N + 9]
     base = filled_cache(2, 2, 2, N + B, d, lens, seed=61, dup_fraction=0.1)
     results = []
-    for small in ("1", "0"):
-        monkeypatch.setenv("VD_SMALL_PATH", small)
+    for kernel in ("small_evict_kernel", other):
+        on_kernel(kernel, monkeypatch)
         c = vd.Cache(base.k.clone(), base.v.clone(), base.len.clone())
         kept = torch.full(c.unit_shape() + (N,), -7, dtype=torch.int32, device="cuda")
         sc = torch.full(c.unit_shape() + (N + B,), float("nan"), device="cuda")
-        vd.vd_evict_block(c, N, None, B, var, vd.VD_MU_RECOMPUTE, None, kept, sc)
+
+        def event():
+            vd.vd_evict_block(c, N, None, B, var, vd.VD_MU_RECOMPUTE, None, kept, sc)
+
+        assert [k for k, _ in evictions(event)] == [kernel]
+        event()
         assert vd.vd_get_device_status() == 0
         results.append((c, kept.view(c.units, N).cpu().numpy(), sc.view(c.units, -1).cpu().numpy()))
     (c1, k1, s1), (c2, k2, s2) = results
@@ -172,14 +186,15 @@ def test_agrees_with_the_fused_kernel(orc, var, monkeypatch):
                                units_view(c2.k)[u, :N].view(torch.int16))
 
 
-def test_tiny_prefill_every_event_both_kernels(orc, monkeypatch):
-    """The smallest workload, every event, with and without the short-cache
-    kernel: identical kept lists and caches (no near ties in this stream)."""
+@pytest.mark.parametrize("other", ["evict_kernel", "resident_evict_kernel"])
+def test_tiny_prefill_every_event_both_kernels(orc, other, monkeypatch):
+    """The smallest workload, every event, in the short-cache kernel and in
+    another: identical kept lists and caches (no near ties in this stream)."""
     _, cfg = wl.config("tiny_prefill")
     d, N, B, T = cfg["head_dim"], cfg["N"], cfg["B"], cfg["T"]
     caches = []
-    for small in ("1", "0"):
-        monkeypatch.setenv("VD_SMALL_PATH", small)
+    for kernel in ("small_evict_kernel", other):
+        on_kernel(kernel, monkeypatch)
         cache = vd.Cache.empty(1, 1, 2, N + B, d)
         st = wl.stream_for(cfg)
         rs = torch.zeros(cache.unit_shape() + (d,), dtype=torch.float64, device="cuda")
@@ -188,9 +203,14 @@ def test_tiny_prefill_every_event_both_kernels(orc, monkeypatch):
             k, v = st.next(B)
             us = cache.unit_shape()
             kept = torch.full(us + (N,), -7, dtype=torch.int32, device="cuda")
-            vd.vd_append_evict_block(cache, k.view(us + (B, d)).contiguous(),
-                                     v.view(us + (B, d)).contiguous(), B, N, None,
-                                     vd.VD_SCORE_L2, vd.VD_MU_RUNNING, rs, kept_idx_out=kept)
+            new = [t.view(us + (B, d)).contiguous() for t in (k, v)]
+
+            def event():
+                vd.vd_append_evict_block(cache, *new, B, N, None, vd.VD_SCORE_L2,
+                                         vd.VD_MU_RUNNING, rs, kept_idx_out=kept)
+
+            assert [k for k, _ in evictions(event)] == [kernel]
+            event()
             kept_all.append(kept.clone())
         assert vd.vd_get_device_status() == 0
         caches.append((cache, kept_all, rs))
@@ -203,7 +223,7 @@ def test_tiny_prefill_every_event_both_kernels(orc, monkeypatch):
 
 
 # ---------------------------------------------------------------------------
-# anomalies: the same status codes as the fused kernel, lengths untouched
+# anomalies: the same status codes as the streaming kernel, lengths untouched
 # ---------------------------------------------------------------------------
 def test_decode_over_budget_and_bad_length():
     d, N = 64, 40

@@ -24,7 +24,7 @@ import oracle
 import paper_2609_23314_gb300 as vd
 from paper_2609_23314_gb300 import build, workloads as wl
 from test_gpu_holefill import run_event
-from vd_gpu import bits, check_scores, new_cache, units_view
+from vd_gpu import bits, check_scores, evictions, new_cache, units_view
 
 pytestmark = pytest.mark.gpu
 VARS = [oracle.L2, oracle.DIR, oracle.NORM]
@@ -188,7 +188,8 @@ def test_split_equals_unsplit_unitwise(case, var, mu):
 @pytest.mark.parametrize("var", VARS, ids=VAR_IDS)
 def test_automatic_split_holefill_against_oracle(orc, var):
     """More units than SMs, one wave at one CTA per unit: the automatic plan
-    splits the launch.  Every unit checked against the oracle through token
+    splits the launch (of the streaming kernel: the resident one would take
+    units of this size).  Every unit checked against the oracle through token
     positions, with the running mean."""
     props = torch.cuda.get_device_properties(0)
     sms = props.multi_processor_count
@@ -203,9 +204,12 @@ def test_automatic_split_holefill_against_oracle(orc, var):
     cache.len.fill_(N)                       # the running sum of the rows before the block
     vd.vd_running_sum_init(cache, rs)
     cache.len.fill_(cap)
-    with env(VD_CLUSTER_SIZE=None, VD_SOLO_UNITS=None, VD_SPLIT_LAUNCH=None):
-        run_event(orc, var, cache, pos, torch.tensor([N], dtype=torch.int32, device="cuda"),
-                  N, B, vd.VD_MU_RUNNING, rs)
+    first = torch.tensor([N], dtype=torch.int32, device="cuda")
+    with env(VD_CLUSTER_SIZE=None, VD_SOLO_UNITS=None, VD_SPLIT_LAUNCH=None, VD_RESIDENT="0"):
+        took = evictions(lambda: vd.vd_evict_block_holefill(cache, N, pos, first, None, B, var,
+                                                            vd.VD_MU_RUNNING, rs))
+        assert [k for k, _ in took] == ["evict_kernel"] * 2 and took[0][1] == sms, took
+        run_event(orc, var, cache, pos, first, N, B, vd.VD_MU_RUNNING, rs)
     ref = torch.zeros_like(rs)
     vd.vd_running_sum_init(cache, ref)
     assert torch.max(torch.abs(ref - rs)).item() <= 1e-9
@@ -221,6 +225,8 @@ def test_automatic_split_score_pass_against_oracle(orc, var):
     U = cache.units
     sc = torch.full(cache.unit_shape() + (cap,), float("nan"), device="cuda")
     with env(VD_CLUSTER_SIZE=None, VD_SOLO_UNITS=None, VD_SPLIT_LAUNCH=None):
+        took = evictions(lambda: vd.vd_score(cache, var, sc))
+        assert [k for k, _ in took] == ["evict_kernel"] * 2, took
         vd.vd_score(cache, var, sc)
     assert vd.vd_get_device_status() == 0
     v = bits(units_view(cache.v))

@@ -18,6 +18,7 @@ and rule (``record_error``); the session prints the table at the end.
 """
 from __future__ import annotations
 
+import ctypes
 import os
 
 import numpy as np
@@ -60,6 +61,66 @@ def record_error(var, s_gpu, s_ora, tag: str = "", tol=None):
     w[0] = max(w[0], rel)
     w[1] = max(w[1], frac)
     w[2] += int(s_ora.size)
+
+
+class _KernelNode(ctypes.Structure):  # CUDA_KERNEL_NODE_PARAMS_v2
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3),
+                ("block", ctypes.c_uint * 3), ("smem", ctypes.c_uint),
+                ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def launched_kernels(call) -> list:
+    """(name, CTAs) of every kernel that call() launches on the current stream,
+    from a stream capture: nothing runs.  The name is the C++ one without
+    namespace and template arguments."""
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def check(code):
+        assert code == 0, f"CUDA driver error {code}"
+
+    stream = torch.cuda.Stream()
+    handle, graph, n = ctypes.c_void_p(stream.cuda_stream), ctypes.c_void_p(), ctypes.c_size_t()
+    with torch.cuda.stream(stream):
+        check(cu.cuStreamBeginCapture_v2(handle, 2))  # relaxed
+        try:
+            call()
+        finally:
+            check(cu.cuStreamEndCapture(handle, ctypes.byref(graph)))
+    check(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    check(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    out = []
+    for node in nodes:
+        kind = ctypes.c_int(-1)
+        check(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value != 0:  # a kernel
+            continue
+        p, name = _KernelNode(), ctypes.c_char_p()
+        check(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+        if p.func:
+            check(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)))
+        else:
+            check(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)))
+        out.append((_plain_name(name.value.decode()), p.grid[0] * p.grid[1] * p.grid[2]))
+    check(cu.cuGraphDestroy(graph))
+    return out
+
+
+def _plain_name(mangled: str) -> str:
+    """_ZN2vd12evict_kernelILi0E... -> evict_kernel; _Z16vd_append_kernelP... ->
+    vd_append_kernel."""
+    rest, name = mangled.removeprefix("_ZN").removeprefix("_Z"), mangled
+    while rest[:1].isdigit():
+        digits = len(rest) - len(rest.lstrip("0123456789"))
+        size = int(rest[:digits])
+        name, rest = rest[digits:digits + size], rest[digits + size:]
+    return name
+
+
+def evictions(call) -> list:
+    """launched_kernels without the appends and the length updates."""
+    return [k for k in launched_kernels(call) if not k[0].startswith("vd_")]
 
 
 def bits(t: torch.Tensor) -> np.ndarray:
