@@ -390,6 +390,11 @@ bool cluster_allowed(int c, int d) {
 // units C = 4 282 us, C = 1 313).  Hole-fill decode and score-only with more
 // units: C = 1 up to one wave, else the smallest C with two waves.
 //
+// The lines are fitted at d = 128 where no other head dim is named.  Elsewhere,
+// ordered block, the rule's C and the others: d = 64, 288 units, n = 1152 C = 1
+// 42.9 (C = 2 40.8, C = 4 59), n = 2176 C = 1 72.2 (C = 2 73.7, C = 4 81); d = 256,
+// 192 units, n = 1152 C = 2 97 (C = 1 107, C = 4 117).
+//
 // Hole-fill block eviction (moves few rows, so the select's cluster
 // synchronisation dominates and grows with C): the smallest C with at least
 // 0.4 of a wave (one short wave beats a long tail and more cluster barriers:
@@ -607,8 +612,9 @@ vd_status launch_dependent(unsigned blocks, cudaStream_t s, void (*kern)(Params.
 // groups clusters of c CTAs: the streaming and resident kernels' grids are units x
 // c CTAs (a cluster per unit), the short-cache kernel's n_seq x units_per_seq (a
 // cluster per sequence, a CTA per unit) or units x 1.
+// A programmatic dependent launch: the kernel waits in griddepcontrol.wait.
 vd_status launch(const void* kern, long long groups, int c, size_t smem, const void* params,
-                 cudaStream_t s, bool dependent = false) {
+                 cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)(groups * c));
   cfg.blockDim = dim3(kThreads);
@@ -619,11 +625,10 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
   attr[0].val.clusterDim.x = (unsigned)c;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  // a programmatic dependent launch (the kernel waits in griddepcontrol.wait)
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = dependent ? 2 : 1;
+  cfg.numAttrs = 2;
   void* args[] = {const_cast<void*>(params)};
   if (cudaLaunchKernelExC(&cfg, kern, args) != cudaSuccess) {
     cudaGetLastError();
@@ -636,25 +641,29 @@ vd_status launch(const void* kern, long long groups, int c, size_t smem, const v
 // clusters all run at once: it is bound by the latency of its phases, so it
 // wins where the streaming kernel has too few rows per SM to hide its own, and
 // loses once several waves of clusters follow one another (288 units of 2176
-// rows, d = 128: 167 us against 136).  C is the largest size, up to 12, that
+// rows, d = 128: 176 us against 130).  C is the largest size, up to 12, that
 // leaves a CTA at least 64 rows and the launch at most two CTAs per SM (decode,
-// which has fewer phases: three), and whose clusters form one wave.  Measured, streaming / resident, d = 128,
-// n = 2176: 8 units 24.9 / 18.2 us (C = 12; C = 8 1.3 us more), 16 units 27.3 /
-// 21.5 (C = 10), 32 units 30.6 / 29.0 (C = 8; C = 4 1.3 us more); n = 1152: 96
-// units 34.4 / 33.7 (C = 3; C = 4, 2.5 CTAs per SM, 50.3).  Both tensors get a
-// buffer where that keeps the wave (8 units 17.6 us in the kernel against
-// 20.3).  More units, or larger ones: C = 1 where three CTAs share an SM (decode:
+// which has fewer phases: three), and whose clusters form one wave.  us,
+// streaming / resident, d = 128, n = 2176: 8 units 25.1 / 18.7 (C = 12; C = 8
+// 21.7), 16 units 27.8 / 22.2 (C = 10; C = 8 23.8), 32 units 31.2 / 29.1 (C = 8; C
+// = 4 30.5); n = 1152, 96 units 34.8 / 33.6 (C = 3; C = 4, 2.5 CTAs per SM, 48.8);
+// d = 64, n = 2176, 32 units 24.4 / 20.6, 64 units 28.6 / 27.8.  Both tensors get a
+// buffer where that keeps the wave (8 units 19.2, else 19.8).  More units, or
+// larger ones: C = 1 where three CTAs share an SM (decode:
 // two), in any number of waves, since a small unit is only its phases in either
-// kernel.  us, streaming / resident: d = 64, 340 rows, 320 units 26.8 / 22.4, 4800
+// kernel: d = 64, 340 rows, 320 units 26.8 / 22.4, 4800
 // units 208 / 182; d = 96, 240 rows, 1600 units 105 / 86 (340 rows, two CTAs per
 // SM, 110 / 127); decode, d = 128, 301 rows, 640 units 42.9 / 33.7, 4800 units
 // 197 / 172 (451 rows, one CTA per SM, 249 / 328).  A hole-fill block event moves
-// so few rows that the streaming kernel catches up at 12 MB of scored rows (d =
-// 256, 1128 rows, 16 units 23.4 / 23.1, 24 units 24.6 / 27.5); otherwise the same
-// lines: hole-fill block, d = 128, 2176 rows, 8 units 20.6 / 17.9, 230 rows, 320
+// so few rows that the streaming kernel catches up at 12 MB of scored rows: n =
+// 2176, d = 128, 16 units (8.9 MB) 22.7 / 21.4, 24 units (13.4 MB) 23.8 / 25.2; d =
+// 64, 40 units (11 MB) 21.8 / 21.4, 48 units (13 MB) 22.1 / 23.3; n = 1128, d =
+// 256, 16 units (9.2 MB) 23.6 / 23.4, 24 units (14 MB) 24.8 / 28.3.  Otherwise the
+// same lines: hole-fill block, d = 128, 2176 rows, 8 units 20.6 / 17.9, 230 rows, 320
 // units 39.1 / 20.1; hole-fill decode, 4097 rows, 8 units 19.2 / 11.0, 201 rows,
-// 4800 units 138 / 86.  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces clusters of
-// c CTAs (100 + c: with both buffers), for tests.  Returns C, or 0.
+// 4800 units 138 / 86.  VD_RESIDENT=0 turns the kernel off, VD_RESIDENT=c forces
+// clusters of c CTAs (100 + c: with both buffers), for tests; a size that cannot
+// run falls back to the streaming kernel.  Returns C, or 0.
 constexpr int kResidentMinRows = 64;
 
 int resident_plan(const void* kern, const PlanKey& k, bool decode, bool holefill,
@@ -800,11 +809,11 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     a.cluster = a.units_per_seq;
     if (a.cluster <= 16 && units <= st->sms && cached_fits(sk, c->n_seq, a.cluster, ssmem, *st)) {
       const vd::SmallArgs sa{a, (int32_t)units, 1};
-      return launch(sk, c->n_seq, a.cluster, ssmem, &sa, s, true);
+      return launch(sk, c->n_seq, a.cluster, ssmem, &sa, s);
     }
     a.cluster = 1;
     const vd::SmallArgs sa{a, (int32_t)units, 0};
-    r = launch(sk, units, 1, ssmem, &sa, s, true);
+    r = launch(sk, units, 1, ssmem, &sa, s);
     return r != VD_OK ? r : clamp_lengths();
   }
   const bool cluster_env = std::getenv("VD_CLUSTER_SIZE") != nullptr;
@@ -832,7 +841,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
   const size_t smem = plan.smem;
   if (plan.resident) {
     const vd::ResidentArgs ra{a, plan.both ? 1 : 0};
-    r = launch(rk, units, a.cluster, smem, &ra, s, true);
+    r = launch(rk, units, a.cluster, smem, &ra, s);
     return r != VD_OK ? r : clamp_lengths();
   }
   const long long solo = plan.solo;
@@ -846,7 +855,7 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     a1.let_next = 1;
     const size_t smem1 = vd::smem_layout(c->capacity, 1, kind).total;
     if (smem1 > (size_t)st->smem_optin) return VD_ERR_UNSUPPORTED;
-    r = launch(kern, solo, 1, smem1, &a1, s, true);
+    r = launch(kern, solo, 1, smem1, &a1, s);
     if (r != VD_OK) return r;
     // the second part's per-unit pointers start at unit `solo`
     const size_t rows = (size_t)solo * c->capacity, dd = (size_t)c->head_dim;
@@ -863,9 +872,9 @@ vd_status run(const vd_cache* c, int32_t N, const int32_t* N_dev, int32_t B, vd_
     if (a.disp_out) a.disp_out += solo;
     if (a.k_new) a.k_new += (size_t)solo * a.B * dd;
     if (a.v_new) a.v_new += (size_t)solo * a.B * dd;
-    r = launch(kern, units - solo, a.cluster, smem, &a, s, true);
+    r = launch(kern, units - solo, a.cluster, smem, &a, s);
   } else {
-    r = launch(kern, units, a.cluster, smem, &a, s, true);
+    r = launch(kern, units, a.cluster, smem, &a, s);
   }
   return r != VD_OK || score_only ? r : clamp_lengths();
 }

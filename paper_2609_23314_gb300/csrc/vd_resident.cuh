@@ -13,7 +13,8 @@
 //              itself (no exchange) up to 64 KB of them; recomputed: column
 //              sums of the slice, exchanged through distributed shared memory
 //   3. score   chunk by chunk as the copies land, with the operations of the
-//              streaming kernel in its order: bit-identical scores
+//              streaming kernel in its order: the same bits for the same mean
+//              (whose sums are added in another order; its remainder may differ)
 //   4. select  every CTA gets every key (16-byte remote stores) and finds the
 //              threshold by itself: one histogram of 1024 buckets over the
 //              range the keys span, then a rank among the threshold's bucket
@@ -28,15 +29,16 @@
 //              fit, and written after one more barrier.  Hole-fill layout:
 //              only the movers are copied, from global memory into the holes.
 //
-// What bounds it: the latency of these steps, each of which runs once.  At 8
-// units of 2176 rows, d = 128 (C = 12) a call takes 19.6 us, 29.0 with the
-// streaming kernel; ncu counts half of the warps' stalls as instruction fetch
-// (no loop repeats often enough to stay cached).  8 warps per CTA beat 16 (17.9
-// us against 19.6 on one box), and rolling the loops up lost 0.8 us: the loads
+// What bounds it: the latency of these steps, each of which runs once; ncu
+// counts half of the warps' stalls as instruction fetch (no loop repeats often
+// enough to stay cached).  us per fused call, calls back to back, streaming /
+// this kernel: 8 units of 2176 rows, d = 128 (C = 12) 25.1 / 18.7 (19.5 with
+// inputs that rotate), recomputed mean 26.0 / 17.4, Dir 29.1 / 20.8, d = 96 30.8 /
+// 19.2; decode, 8 units of 4097 rows 22.8 / 13.4.  8 warps per CTA beat 16 (17.9
+// us in the kernel against 19.6), and rolling the loops up lost 0.8 us: the loads
 // that an unrolled loop keeps in flight count for more.  The barriers that
 // only order execution are relaxed arrivals: the release form waited 2 to 5 us
-// for the bulk copies in flight.  Recomputed mean at 8 units: 35.0 -> 26.5 us;
-// Dir 35.5 -> 21.8; d = 96 32.9 -> 17.5; decode, 4097 rows 25.5 -> 16.1.
+// for the bulk copies in flight.
 #pragma once
 
 #include <climits>

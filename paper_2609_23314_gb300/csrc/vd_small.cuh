@@ -1,5 +1,5 @@
 // vd_small.cuh -- pi_N of Sec. 2.1 Eq. (eviction) for short caches, where the
-// fused kernel's machinery (multi-pass radix select, streaming rings, the
+// streaming kernel's machinery (multi-pass radix select, streaming rings, the
 // separate length update) costs more than the work itself.
 //
 // One CTA per (sequence, layer, KV head) unit.  In a launch of few units the
@@ -12,7 +12,7 @@
 //   1. mean    double-float column sums (running mode: the caller's fp64 sum
 //              S plus the appended rows), kept as an fp32 part and remainder
 //   2. score   L2 ((v - hi) - lo)^2, Dir |w|^2 / (2 |v|^2) with
-//              w = v - (|v|/|m|) m, Norm |v|^2, as in the fused kernel
+//              w = v - (|v|/|m|) m, Norm |v|^2, as in the streaming kernel
 //   3. select  decode: an arg-min over (key, -slot); block:
 //              rank_j = #{i : key_i > key_j} + #{i < j : key_i == key_j}, row
 //              j survives iff rank_j < N (Eq. eviction, ties to the lower
@@ -32,7 +32,7 @@
 // 128, 128 rows, 320 units 23.7 / 15.7, 1600 units 64 / 42, 4800 units 179 / 108;
 // decode, 101 rows, 1600 units 50 / 29.
 //
-// Same validation, outputs and status codes as the fused kernel; no hole-fill
+// Same validation, outputs and status codes as the streaming kernel; no hole-fill
 // layout and no sigma (those calls take the other kernels).
 #pragma once
 
@@ -101,7 +101,7 @@ __device__ __forceinline__ ff small_column_sum(int d, int count, RowOf row_of, S
   return t;
 }
 
-// The kernel's parameters: the fused kernel's, plus the number of units.
+// The kernel's parameters: the streaming kernel's, plus the number of units.
 struct SmallArgs {
   EvictArgs e;
   int32_t n_units;  // n_seq * units_per_seq: the grid's CTAs
@@ -111,7 +111,8 @@ struct SmallArgs {
 // VAR: 0 L2, 1 Dir, 2 Norm.  DECODE: the decode entry points (n <= N + 1);
 // the selection is the same.  FUSED: rows at or above len come from the
 // caller's staging buffers (the append of Eq. block_processing).
-// a.cluster = units per sequence (the cluster size), a.capacity <= kSmallMaxRows.
+// a.cluster: the cluster size, with set_len the units per sequence, else 1.
+// a.capacity <= kSmallMaxRows.
 template <int VAR, bool DECODE, bool FUSED>
 __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArgs sa) {
   const EvictArgs& a = sa.e;
@@ -157,7 +158,7 @@ __global__ void __launch_bounds__(kThreads, 1) small_evict_kernel(const SmallArg
   const uint16_t* knu = FUSED ? (a.score_k ? a.v_new : a.k_new) + (size_t)u * a.B * d : nullptr;
   const uint16_t* vnu = FUSED ? (a.score_k ? a.k_new : a.v_new) + (size_t)u * a.B * d : nullptr;
 
-  // ---- validation: the same per-sequence checks as the fused kernel -------
+  // ---- validation: the same per-sequence checks as the streaming kernel -------
   bool ok = unit_ok;
   if (!unit_ok) {
     if (tid == 0) record_status(a.status, kStInternal);
